@@ -110,10 +110,13 @@ typedef struct {
                          are stored colour-split, each row's red cells
                          before its black ones, so that a pass reads only
                          its own colour of them) */
-    int coarse_cells; /* levels of at most this many cells run inside one CTA
-                         per box (the coarse end of the V-cycle as a single
-                         launch); 0 default (4096 in FP32 V-cycles, 1024 in
-                         FP64 ones, whose FP64 rate per SM is low), -1 off */
+    int coarse_cells; /* the coarse end of the V-cycle runs as a single launch, one
+                         thread-block cluster per box with its levels in shared
+                         memory: every level of at most this many cells (as far
+                         as they fit).  0 default: 4096 in FP32 V-cycles, 1024
+                         in FP64 ones, and below the finest level also larger
+                         levels while a pass costs less there than its launch
+                         would; -1 off */
     int inner_cycles; /* MG_MIXED: FP32 V-cycles per FP64 refinement step.
                          1..8: that many.  0 (default): adaptive, up to 8:
                          the step solves A e = r32 for a scaled copy r32 of

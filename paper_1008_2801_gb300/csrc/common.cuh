@@ -209,8 +209,6 @@ struct SetupBox {
 };
 typedef DescSet<SetupBox> SetupSet;
 
-// The coarse end of one box's V-cycle, run by a single CTA: levels
-// lv[0] (the first level small enough) down to lv[nlev-1] (the coarsest).
 // Ghost exchange of a coupled level: copy the src box's cells of a patch
 // (extents ex, ey, ez; one of them 1) into the dst box's guard cells (local
 // coordinates, guard positions -1 or n).  Box indices refer to the level's
@@ -234,15 +232,30 @@ struct UnionBottom {
 };
 
 constexpr int kMaxCoarse = 10;
+constexpr int kTailSolo = 1024;              // most cells of a level run by one CTA of a cluster
+constexpr int kTailSmem = 227 * 1024 - 4096; // dynamic shared memory of a cluster's CTA (the job
+                                             // descriptor is static)
+// Where a level of the cluster's coarse V-cycle sits in a CTA's shared memory:
+// offsets in elements of phi (with guards), f, the weights and 1/D (dense).
+struct TailLevel {
+    int phi, f, wx, wy, wz, inv;
+    int dg;         // stored D (FP64), -1: read from global memory
+    int hp;         // f, 1/D and D rows: elements of a colour's half (colour-split levels), 0: natural
+    int red;        // restrict the residual of the red children only
+};
+// Coarse end of one box's V-cycle: levels lv[0] down to lv[nlev-1] (the
+// coarsest), the first ndist of them split over the cluster by planes.
 template <class T>
 struct CoarseJob {
     int nlev;
     int box;
+    int ndist;
+    int nzc;        // planes of level ndist - 1 (the coarsest split level)
+    int per;        // bits 0-2: x, y, z axis periodic
+    int scratch;    // offset: residuals of the coarsest split level (first CTA)
+    int ainv;       // offset: dense coarsest inverse (first CTA), -1: in global memory
+    TailLevel tl[kMaxCoarse];
     Box<T> lv[kMaxCoarse];
-    // periodic axes: the level's self-exchange records (copied into the
-    // box's own guard cells before every pass and residual), else 0
-    const ExchRec *rec[kMaxCoarse];
-    int nrec[kMaxCoarse];
 };
 
 // Per-box convergence state of a solve, kept on the device so that the

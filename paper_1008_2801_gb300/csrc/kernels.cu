@@ -13,10 +13,13 @@
 #include "kernels.h"
 
 #include <algorithm>
+#include <cooperative_groups.h>
 #include <type_traits>
 
 #include <atomic>
 #include <mutex>
+
+namespace cg = cooperative_groups;
 
 namespace mg {
 
@@ -841,166 +844,401 @@ __global__ void __launch_bounds__(kThreads) k_bottom(BoxSet<T> S, const int *__r
     }
 }
 
-// --------------------------------------------- coarse V-cycle in one CTA ----
+// ------------------------------------- coarse V-cycle in one cluster per box ----
 //
-// Levels of a few thousand cells take microseconds of work but a kernel
-// launch each; the coarse end of every box's V-cycle therefore runs inside
-// one CTA per box, with block barriers between stages: nu1 red/black passes
-// and residual + restriction going down, the dense coarsest solve, then
-// prolongation and nu2 passes going up.  Same stage definitions as the
-// per-level kernels; data stay in global memory (L1/L2 resident).
+// Levels of a few ten thousand cells take well under a microsecond of work a
+// stage, but a launch each; the coarse end of every box's V-cycle therefore
+// runs inside one thread-block cluster per box, with its levels in shared
+// memory from the first pass to the last: nu1 red/black passes and residual +
+// restriction going down, the dense coarsest solve, then prolongation and nu2
+// passes going up.  Same stage definitions and per-cell arithmetic as the
+// per-level kernels (bitwise the same results).
+//
+// The first ndist levels are split over the cluster by planes of z (every
+// level's split halves with the planes, so a fine pair of planes and its
+// coarse plane sit in one CTA); a CTA's boundary planes are stored into the
+// neighbour's halo plane as they are updated (distributed shared memory), and
+// one cluster barrier ends each pass.  The levels below (at most kTailSolo
+// cells) run in the cluster's first CTA alone, where a block barrier does.
+// What bounds it: the dependent chain of about 20 stages per two levels, each
+// a barrier (~0.3 us), the shared-memory latency and, in FP64, the narrow pipe
+// (16 cycles an SM per warp instruction: 1.7 us for a pass over 32^3 on 16
+// SMs; a chain of 7 dependent FP64 operations alone is 0.4 us).  Weights are
+// loaded before the wait on the preceding kernel.  FP64, 32^3 and below: 60 us
+// a cycle against 93 us as launches plus a one-CTA kernel below 16^3 that
+// worked on global memory (the 64^3 solve 1.76 -> 1.51 ms).
 
-// FP32: 1024 threads; FP64: 512 (its register footprint is larger)
-template <class T>
-struct CoarseThreads { static constexpr int value = sizeof(T) == 8 ? 512 : 1024; };
+constexpr int kTailThreads = 512;
 
+// One level of a CTA's part, in shared memory (offsets from the host's plan).
+// f, 1/D and D keep the level's colour split: hp > 0: a row holds its red
+// cells, then (from hp) its black ones; hp = 0: in x order.
 template <class T>
-__device__ __forceinline__ void cta_pass(const Box<T> &B, int color)
-{
-    const int npx = (B.nx + 1) >> 1;
-    const int tot = npx * B.ny * B.nz;
-    for (int q = threadIdx.x; q < tot; q += CoarseThreads<T>::value) {
-        const int p = q % npx;
-        const int r = q / npx;
-        const int j = r % B.ny, k = r / B.ny;
-        const int i = 2 * p + ((j + k + color + B.par) & 1);
-        if (i >= B.nx) continue;
-        const long long c = (long long)k * B.Q + (long long)j * B.P + i;
-        const long long cf =
-            split_on(B) ? (long long)k * B.Q + (long long)j * B.P + (color ? (B.P >> 1) : 0) + p
-                        : c;
-        B.phi[c] = gs_value<T>(B.phi, B.f, B.invD, B.wx, B.wy, B.wz, c, cf, B.P, B.Q);
+struct TailView {
+    T *phi, *f;                  // phi: [np + 2][ny + 2][nx + 2]; f: [np][ny][fp]
+    const T *wx, *wy, *wz;       // [np][ny][nx + 2], [np][ny + 1][nx], [np + 1][ny][nx]
+    const T *inv, *dg;           // [np][ny][fp]; dg NULL: D is read from global memory
+    int nx, ny, p, q, np, z0, par, fp, hp;
+    int lo, hi, lo_top;          // ranks that own planes z0 - 1 and z0 + np (-1: a wall); halo plane of lo
+};
+
+// u / n for 0 <= u < 2^20, n >= 1 and rn = 1.0f / n: (u + 1/2) / n lies at
+// least 1 / (2n) from an integer, further than the two FP32 roundings reach
+// (an integer division is a chain of about 100 cycles, paid at every stage).
+__device__ __forceinline__ int tail_div(int u, float rn) { return (int)(((float)u + 0.5f) * rn); }
+
+// This thread's walk over [0, ex) x [0, ey) x [0, ez) in steps of the CTA.
+struct TailWalk {
+    int x, y, z, sx, sy, sz, ex, ey, ez;
+    __device__ __forceinline__ TailWalk(int ex_, int ey_, int ez_) : ex(ex_), ey(ey_), ez(ez_)
+    {
+        const float rx = __frcp_rn((float)ex), ry = __frcp_rn((float)ey);
+        const int u = threadIdx.x, r = tail_div(u, rx), r2 = tail_div(kTailThreads, rx);
+        x = u - r * ex;
+        z = tail_div(r, ry);
+        y = r - z * ey;
+        sx = kTailThreads - r2 * ex;
+        sz = tail_div(r2, ry);
+        sy = r2 - sz * ey;
     }
-}
-
-// Periodic axes: fill the box's guard cells from its own opposite faces
-// (records whose source is the box itself); the caller synchronises.
-template <class T>
-__device__ __forceinline__ void cta_exchange(const Box<T> &B, const ExchRec *rec, int nrec)
-{
-    for (int q = 0; q < nrec; ++q) {
-        const ExchRec R = rec[q];
-        const int n = R.ex * R.ey * R.ez;
-        for (int e = threadIdx.x; e < n; e += CoarseThreads<T>::value) {
-            const int a = e % R.ex, r = e / R.ex;
-            const int bb = r % R.ey, c = r / R.ey;
-            B.phi[(long long)(R.dk + c) * B.Q + (long long)(R.dj + bb) * B.P + R.di + a] =
-                B.phi[(long long)(R.sk + c) * B.Q + (long long)(R.sj + bb) * B.P + R.si + a];
+    template <class F>
+    __device__ __forceinline__ void each(F fn) const
+    {
+        int a = x, b = y, c = z;
+        while (c < ez) {
+            fn(a, b, c);
+            a += sx;
+            b += sy;
+            c += sz;
+            if (a >= ex) { a -= ex; ++b; }
+            if (b >= ey) { b -= ey; ++c; }
         }
     }
+};
+
+// N elements global -> shared (both aligned to N elements) without a register
+// or a wait (tail_async_wait)
+template <int N, class T>
+__device__ __forceinline__ void tail_async(T *dst, const T *src)
+{
+    constexpr int bytes = N * (int)sizeof(T);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src), "n"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void tail_async_wait()
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 template <class T>
-__device__ __forceinline__ void cta_resid_restrict(const Box<T> &B)
+__device__ __forceinline__ int tail_at(const TailView<T> &V, int i, int j, int z)
 {
-    const int cx = B.nx / 2, cy = B.ny / 2, cz = B.nz / 2;
-    const int tot = cx * cy * cz;
-    for (int q = threadIdx.x; q < tot; q += CoarseThreads<T>::value) {
-        const int I = q % cx, r = q / cx;
-        const int J = r % cy, K = r / cy;
-        auto children = [&](auto has_d) {
-            constexpr bool HD = decltype(has_d)::value;
-            T sum = T(0);
-            for (int c = 0; c < 2; ++c)
-                for (int bb = 0; bb < 2; ++bb)
-                    for (int a = 0; a < 2; ++a) {
-                        const long long g = (long long)(2 * K + c) * B.Q +
-                                            (long long)(2 * J + bb) * B.P + 2 * I + a;
-                        sum += residual_at<T, HD>(B.phi, B.f, B.wx, B.wy, B.wz, B.D, g,
-                                                  fidx(B, 2 * I + a, 2 * J + bb, 2 * K + c),
-                                                  B.P, B.Q);
-                    }
-            return sum;
-        };
-        const T sum = B.D ? children(std::true_type{}) : children(std::false_type{});
-        const long long cc = (long long)K * B.cQ + (long long)J * B.cP + I;
-        B.fc[cfidx(B, I, J, K)] = sum * T(0.125);
-        B.phic[cc] = T(0);
+    return (z + 1) * V.q + (j + 1) * V.p + i + 1;
+}
+// element of f, 1/D and D
+template <class T>
+__device__ __forceinline__ int tail_fat(const TailView<T> &V, int i, int j, int z)
+{
+    const int r = (z * V.ny + j) * V.fp;
+    return V.hp ? r + (((i + j + V.z0 + z + V.par) & 1) ? V.hp : 0) + (i >> 1) : r + i;
+}
+
+// v into the copies of cell (i, j, z): neighbouring CTAs' halo planes and, on
+// periodic axes, the guard cells
+template <class T>
+__device__ __forceinline__ void tail_push(const cg::cluster_group &cl, const TailView<T> &V, int per,
+                                          int i, int j, int z, int c, T v)
+{
+    if (z == 0 && V.lo >= 0)
+        cl.map_shared_rank(V.phi, V.lo)[V.lo_top * V.q + (j + 1) * V.p + i + 1] = v;
+    if (z == V.np - 1 && V.hi >= 0)
+        cl.map_shared_rank(V.phi, V.hi)[(j + 1) * V.p + i + 1] = v;
+    if (per & 1) {
+        if (i == 0) V.phi[c + V.nx] = v;
+        if (i == V.nx - 1) V.phi[c - V.nx] = v;
+    }
+    if (per & 2) {
+        if (j == 0) V.phi[c + V.ny * V.p] = v;
+        if (j == V.ny - 1) V.phi[c - V.ny * V.p] = v;
     }
 }
 
 template <class T>
-__device__ __forceinline__ void cta_prolong(const Box<T> &B)
+__global__ void __launch_bounds__(kTailThreads, 1)
+    k_coarse_vcycle(const CoarseJob<T> *__restrict__ jobs, const int *__restrict__ active, int nu1,
+                    int nu2, int post_first, int zero_start)
 {
-    const int tot = B.nx * B.ny * B.nz;
-    for (int q = threadIdx.x; q < tot; q += CoarseThreads<T>::value) {
-        const int i = q % B.nx, r = q / B.nx;
-        const int j = r % B.ny, k = r / B.ny;
-        const long long c = (long long)k * B.Q + (long long)j * B.P + i;
-        B.phi[c] += B.phic[(long long)(k >> 1) * B.cQ + (long long)(j >> 1) * B.cP + (i >> 1)];
-    }
-}
-
-template <class T>
-__device__ __forceinline__ void cta_bottom(const Box<T> &B, T *fs)
-{
-    const int nx = B.nx, ny = B.ny, n = nx * ny * B.nz;
-    for (int q = threadIdx.x; q < n; q += CoarseThreads<T>::value) {
-        const int i = q % nx, j = (q / nx) % ny, k = q / (nx * ny);
-        fs[q] = B.f[fidx(B, i, j, k)];
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int r = warp; r < n; r += CoarseThreads<T>::value / 32) {
-        const T *row = B.ainv + (long long)r * n;
-        T acc = T(0);
-        for (int q = lane; q < n; q += 32) acc = fmadd(row[q], fs[q], acc);
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (lane == 0) {
-            const int i = r % nx, j = (r / nx) % ny, k = r / (nx * ny);
-            B.phi[(long long)k * B.Q + (long long)j * B.P + i] = acc;
-        }
-    }
-}
-
-template <class T>
-__global__ void __launch_bounds__(CoarseThreads<T>::value) k_coarse_vcycle(const CoarseJob<T> *__restrict__ jobs,
-                                                                  const int *__restrict__ active,
-                                                                  int nu1, int nu2, int post_first)
-{
-    pdl_wait();
+    extern __shared__ __align__(16) char tail_smem[];
     __shared__ CoarseJob<T> J;
-    __shared__ T fs[MG_BOTTOM_CELLS];
+    __shared__ TailView<T> views[kMaxCoarse];
+    const cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), CL = (int)cl.num_blocks();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    T *const sm = reinterpret_cast<T *>(tail_smem);
     {
         const int words = (int)(sizeof(CoarseJob<T>) / sizeof(int));
-        const int *src = reinterpret_cast<const int *>(jobs + blockIdx.x);
+        const int *src = reinterpret_cast<const int *>(jobs + blockIdx.x / CL);
         int *dst = reinterpret_cast<int *>(&J);
-        for (int w = threadIdx.x; w < words; w += CoarseThreads<T>::value) dst[w] = src[w];
+        for (int w = tid; w < words; w += kTailThreads) dst[w] = src[w];
     }
     __syncthreads();
-    if (active && !active[J.box]) return;  // uniform over the CTA
-    const int nl = J.nlev;
-    auto exch = [&](int l) {
-        if (J.nrec[l] == 0) return;
-        cta_exchange<T>(J.lv[l], J.rec[l], J.nrec[l]);
-        __syncthreads();
-    };
+    const int nl = J.nlev, nd = J.ndist, per = J.per;
+    if (tid < nl) {   // a thread per level
+        const int l = tid;
+        const Box<T> &B = J.lv[l];
+        const TailLevel &L = J.tl[l];
+        auto plane0 = [&](int r) {   // first plane of rank r
+            return l < nd ? ((r * J.nzc) / CL) << (nd - 1 - l) : (r == 0 ? 0 : B.nz);
+        };
+        auto owner = [&](int k) {    // rank of plane k
+            return l < nd ? (((k >> (nd - 1 - l)) + 1) * CL + J.nzc - 1) / J.nzc - 1 : 0;
+        };
+        TailView<T> V;
+        V.nx = B.nx;
+        V.ny = B.ny;
+        V.p = B.nx + 2;
+        V.q = V.p * (B.ny + 2);
+        V.z0 = plane0(rank);
+        V.np = plane0(rank + 1) - V.z0;
+        V.par = B.par;
+        V.hp = L.hp;
+        V.fp = L.hp ? 2 * L.hp : B.nx;
+        V.phi = sm + L.phi;
+        V.f = sm + L.f;
+        V.wx = sm + L.wx;
+        V.wy = sm + L.wy;
+        V.wz = sm + L.wz;
+        V.inv = sm + L.inv;
+        V.dg = L.dg >= 0 ? sm + L.dg : nullptr;
+        V.lo = V.hi = -1;
+        V.lo_top = 0;
+        int kl = V.z0 - 1, kh = V.z0 + V.np;
+        if (per & 4) {
+            if (kl < 0) kl += B.nz;
+            if (kh >= B.nz) kh -= B.nz;
+        }
+        if (kl >= 0) {
+            V.lo = owner(kl);
+            V.lo_top = plane0(V.lo + 1) - plane0(V.lo) + 1;
+        }
+        if (kh < B.nz) V.hi = owner(kh);
+        views[l] = V;
+    }
+    __syncthreads();
+    // the weights of this CTA's planes, before the wait: no kernel of a solve
+    // writes them (pairs of elements; a level that is smoothed has even nx)
     for (int l = 0; l + 1 < nl; ++l) {
-        for (int s = 0; s < nu1; ++s) {
-            exch(l);
-            cta_pass<T>(J.lv[l], 0);
-            __syncthreads();
-            exch(l);
-            cta_pass<T>(J.lv[l], 1);
-            __syncthreads();
-        }
-        exch(l);
-        cta_resid_restrict<T>(J.lv[l]);
-        __syncthreads();
+        const TailView<T> V = views[l];
+        if (V.np == 0) continue;
+        const Box<T> &B = J.lv[l];
+        const long long g0 = (long long)V.z0 * B.Q;
+        const int P = B.P, Q = (int)B.Q, h = V.nx >> 1;
+        const T *const gx = B.wx + g0, *const gy = B.wy + g0, *const gz = B.wz + g0,
+                *const gi = B.invD + g0, *const gd = B.D + g0;
+        T *const sx = const_cast<T *>(V.wx), *const sy = const_cast<T *>(V.wy),
+                 *const sz = const_cast<T *>(V.wz), *const si = const_cast<T *>(V.inv),
+                 *const sd = const_cast<T *>(V.dg);
+        const int hp2 = V.fp >> 1;   // (colour-split rows: the last pair of a half may be padding)
+        TailWalk(h + 1, V.ny + 1, V.np + 1).each([&](int x, int j, int z) {
+            const int r = z * Q + j * P, row = z * V.ny + j;
+            const bool jy = j < V.ny, kz = z < V.np;
+            if (jy && kz) tail_async<2>(sx + row * V.p + 2 * x, gx + r + 2 * x);
+            if (x < h) {
+                const int d = row * V.nx + 2 * x;
+                if (kz) tail_async<2>(sy + d + z * V.nx, gy + r + 2 * x);
+                if (jy) tail_async<2>(sz + d, gz + r + 2 * x);
+            }
+            if (x < hp2 && jy && kz) {
+                const int q = r + (V.hp && 2 * x >= V.hp ? (P >> 1) + 2 * x - V.hp : 2 * x);
+                tail_async<2>(si + row * V.fp + 2 * x, gi + q);
+                if (sd) tail_async<2>(sd + row * V.fp + 2 * x, gd + q);
+            }
+        });
     }
-    cta_bottom<T>(J.lv[nl - 1], fs);
-    __syncthreads();
-    for (int l = nl - 2; l >= 0; --l) {
-        cta_prolong<T>(J.lv[l]);
-        __syncthreads();
-        for (int s = 0; s < nu2; ++s) {
-            exch(l);
-            cta_pass<T>(J.lv[l], post_first);
+    for (int l = 0; l < nl; ++l) {   // phi = 0, guards and halos too
+        const TailView<T> V = views[l];
+        constexpr int N = 16 / (int)sizeof(T);   // (the plan pads every array to 16 bytes)
+        if (V.np > 0)
+            for (int c = N * tid; c < (V.np + 2) * V.q; c += N * kTailThreads)
+                *reinterpret_cast<float4 *>(V.phi + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (J.ainv >= 0 && rank == 0) {
+        const Box<T> &B = J.lv[nl - 1];
+        const int n = B.nx * B.ny * B.nz;
+        for (int q = tid; q < n * n; q += kTailThreads) tail_async<1>(sm + J.ainv + q, B.ainv + q);
+    }
+    pdl_wait();
+    if (active && !active[J.box]) return;  // uniform over the cluster
+    {   // the first level's f (and phi unless it is 0)
+        const Box<T> &B = J.lv[0];
+        const TailView<T> V = views[0];
+        const bool split = split_on(B);
+        TailWalk(V.nx, V.ny, V.np).each([&](int i, int j, int z) {
+            const long long g = (long long)(V.z0 + z) * B.Q + (long long)j * B.P;
+            const int odd = (i + j + V.z0 + z + V.par) & 1;
+            tail_async<1>(V.f + tail_fat(V, i, j, z),
+                          B.f + g + (split ? (odd ? (B.P >> 1) : 0) + (i >> 1) : i));
+            if (!zero_start) tail_async<1>(V.phi + tail_at(V, i, j, z), B.phi + g + i);
+        });
+    }
+    tail_async_wait();
+    if (nd > 0) cl.sync();   // every CTA's halos are zero before a neighbour writes them
+    else __syncthreads();
+    if (!zero_start) {
+        const TailView<T> V = views[0];
+        TailWalk(V.nx, V.ny, V.np).each([&](int i, int j, int z) {
+            const int c = tail_at(V, i, j, z);
+            tail_push(cl, V, per, i, j, z, c, V.phi[c]);
+        });
+        if (nd > 0) cl.sync();
+        else __syncthreads();
+    }
+    // down the levels 0 .. nl - 2, the coarsest, and up again: one copy of
+    // each stage's code (a stage runs a few times a launch, so that its
+    // instruction fetches count)
+    for (int step = 0; step < 2 * nl - 1; ++step) {
+        const bool down = step < nl - 1;
+        const int l = down ? step : 2 * (nl - 1) - step;
+        const bool split = l < nd;
+        if (!down && l == nd - 1) cl.sync();   // the first CTA's correction is there
+        if (!split && rank != 0) continue;
+        const TailView<T> V = views[l];
+        auto sync = [&]() {
+            if (split) cl.sync();
+            else __syncthreads();
+        };
+        if (l == nl - 1) {   // the coarsest level: phi = A^{-1} f, a warp per row
+            const Box<T> &B = J.lv[l];
+            const int n = V.nx * V.ny * B.nz;
+            const float rx = __frcp_rn((float)V.nx), ry = __frcp_rn((float)V.ny);
+            for (int r = warp; r < n; r += kTailThreads / 32) {
+                const T *row = (J.ainv >= 0 ? sm + J.ainv : B.ainv) + (long long)r * n;
+                T acc = T(0);
+                for (int q = lane; q < n; q += 32) acc = fmadd(row[q], V.f[q], acc);
+                for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+                if (lane == 0) {
+                    const int t = tail_div(r, rx), k = tail_div(t, ry);
+                    V.phi[tail_at(V, r - t * V.nx, t - k * V.ny, k)] = acc;
+                }
+            }
             __syncthreads();
-            exch(l);
-            cta_pass<T>(J.lv[l], 1 - post_first);
+            continue;
+        }
+        const int nu = down ? nu1 : nu2, first = down ? 0 : post_first;
+        const TailWalk W(V.nx >> 1, V.ny, V.np);
+        if (!down) {
+            // prolongation: a sweep's first pass reads only the other colour,
+            // so only that colour takes the correction (both when no sweep
+            // follows).  The coarse phi sits in this CTA or in the first.
+            const TailView<T> C = views[l + 1];
+            const bool away = l == nd - 1;
+            const T *const pc = away ? cl.map_shared_rank(C.phi, 0) : C.phi;
+            const int cz0 = away ? 0 : C.z0;
+            W.each([&](int x, int j, int z) {
+                const int k = V.z0 + z;
+                const T e = pc[((k >> 1) - cz0 + 1) * C.q + ((j >> 1) + 1) * C.p + x + 1];
+                for (int a = 0; a < 2; ++a) {
+                    const int i = 2 * x + a;
+                    if (nu2 > 0 && ((i + j + k + V.par) & 1) == post_first) continue;
+                    const int c = tail_at(V, i, j, z);
+                    const T v = V.phi[c] + e;
+                    V.phi[c] = v;
+                    tail_push(cl, V, per, i, j, z, c, v);
+                }
+            });
+            sync();
+        }
+        for (int s = 0; s < 2 * nu; ++s) {
+            const int color = (s & 1) ? 1 - first : first;
+            // phi = 0 on entry: the first pass is -f / D (the chain's value)
+            const bool zero = down && s == 0 && (zero_start || l > 0);
+            W.each([&](int x, int j, int z) {
+                const int i = 2 * x + ((j + V.z0 + z + color + V.par) & 1);
+                const int c = tail_at(V, i, j, z);
+                const int row = z * V.ny + j, d = row * V.nx + i, e = d + z * V.nx;
+                const int fi = row * V.fp + (V.hp ? (color ? V.hp : 0) + x : i);
+                T v = -V.f[fi];
+                if (!zero) {
+                    const T *const wx = V.wx + row * V.p + i;
+                    v = fmadd(wx[0], V.phi[c - 1], v);
+                    v = fmadd(wx[1], V.phi[c + 1], v);
+                    v = fmadd(V.wy[e], V.phi[c - V.p], v);
+                    v = fmadd(V.wy[e + V.nx], V.phi[c + V.p], v);
+                    v = fmadd(V.wz[d], V.phi[c - V.q], v);
+                    v = fmadd(V.wz[d + V.nx * V.ny], V.phi[c + V.q], v);
+                }
+                v *= V.inv[fi];
+                V.phi[c] = v;
+                tail_push(cl, V, per, i, j, z, c, v);
+            });
+            sync();
+        }
+        if (!down) continue;
+        // residuals (of the red cells, or all), each in its cell's place of the
+        // scratch array, then f of level l + 1 by the per-level kernel's sum.
+        // The last split level's go to the first CTA: the two fine planes of a
+        // coarse cell may sit in different CTAs there.
+        const Box<T> &B = J.lv[l];
+        const bool red = J.tl[l].red != 0, away = l == nd - 1;
+        T *const res = away ? cl.map_shared_rank(sm + J.scratch, 0) : sm + J.scratch;
+        const int kb = away ? V.z0 : 0, nr = red ? V.nx >> 1 : V.nx;
+        const T *const gd = B.D;
+        TailWalk(nr, V.ny, V.np).each([&](int x, int j, int z) {
+            const int k = V.z0 + z;
+            const int i = red ? 2 * x + ((j + k + V.par) & 1) : x;
+            const int c = tail_at(V, i, j, z);
+            const int row = z * V.ny + j, d = row * V.nx + i, e = d + z * V.nx;
+            const int fi = tail_fat(V, i, j, z);
+            const T *const wx = V.wx + row * V.p + i;
+            const T a = wx[0], b = wx[1], g = V.wy[e], h = V.wy[e + V.nx], m = V.wz[d],
+                    n = V.wz[d + V.nx * V.ny];
+            T D;
+            if (sizeof(T) == sizeof(float)) D = ((a + b) + (g + h)) + (m + n);
+            else if (V.dg) D = V.dg[fi];
+            else D = gd[fidx(B, i, j, k)];
+            T r = fmadd(D, V.phi[c], V.f[fi]);
+            r = fmadd(-a, V.phi[c - 1], r);
+            r = fmadd(-b, V.phi[c + 1], r);
+            r = fmadd(-g, V.phi[c - V.p], r);
+            r = fmadd(-h, V.phi[c + V.p], r);
+            r = fmadd(-m, V.phi[c - V.q], r);
+            res[((kb + z) * V.ny + j) * nr + x] = fmadd(-n, V.phi[c + V.q], r);
+        });
+        if (away) cl.sync();
+        else __syncthreads();
+        if (!away || rank == 0) {
+            const TailView<T> C = views[l + 1];
+            const T *const src = sm + J.scratch;
+            TailWalk(C.nx, C.ny, away ? J.lv[l + 1].nz : C.np).each([&](int I, int jc, int K) {
+                const T *const r0 = src + (2 * K * V.ny + 2 * jc) * nr, *const r1 = r0 + nr,
+                               *const r2 = r0 + V.ny * nr, *const r3 = r2 + nr;
+                T sum;
+                if (red) {
+                    sum = ((r0[I] + r1[I]) + r2[I]) + r3[I];
+                } else {
+                    sum = T(0) + r0[2 * I];
+                    sum += r0[2 * I + 1];
+                    sum += r1[2 * I];
+                    sum += r1[2 * I + 1];
+                    sum += r2[2 * I];
+                    sum += r2[2 * I + 1];
+                    sum += r3[2 * I];
+                    sum += r3[2 * I + 1];
+                }
+                C.f[tail_fat(C, I, jc, K)] = sum * T(0.125);
+            });
             __syncthreads();
         }
+    }
+    {   // the first level's solution
+        const Box<T> &B = J.lv[0];
+        const TailView<T> V = views[0];
+        TailWalk(V.nx, V.ny, V.np).each([&](int i, int j, int z) {
+            B.phi[(long long)(V.z0 + z) * B.Q + (long long)j * B.P + i] =
+                V.phi[tail_at(V, i, j, z)];
+        });
     }
 }
 
@@ -2883,12 +3121,58 @@ cudaError_t launch_bottom(const BoxSet<T> &S, const int *active, int max_cells, 
 }
 
 template <class T>
-cudaError_t launch_coarse_vcycle(const CoarseJob<T> *jobs, int njobs, const int *active, int nu1,
-                                 int nu2, cudaStream_t st, int post_first)
+int tail_clusters(int cl, size_t smem)
+{
+    void (*const k)(const CoarseJob<T> *, const int *, int, int, int, int) = k_coarse_vcycle<T>;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmem) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cl);
+    cfg.blockDim = dim3(kTailThreads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
+}
+template int tail_clusters<double>(int, size_t);
+template int tail_clusters<float>(int, size_t);
+
+template <class T>
+cudaError_t launch_coarse_vcycle(const CoarseJob<T> *jobs, int njobs, int cl, size_t smem,
+                                 const int *active, int nu1, int nu2, cudaStream_t st,
+                                 int post_first, bool zero_start)
 {
     if (njobs == 0) return cudaSuccess;
-    return pdl_launch(k_coarse_vcycle<T>, dim3(njobs), dim3(CoarseThreads<T>::value), 0, st, jobs,
-                      active, nu1, nu2, post_first);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(njobs * cl);
+    cfg.blockDim = dim3(kTailThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl_enabled() ? 2 : 1;
+    return counted(cudaLaunchKernelEx(&cfg, k_coarse_vcycle<T>, jobs, active, nu1, nu2, post_first,
+                                      zero_start ? 1 : 0));
 }
 
 cudaError_t launch_refine_update(const BoxSet<double> &S64, const BoxSet<float> &S32,
@@ -3292,8 +3576,8 @@ cudaError_t launch_pcg_scalars(int nbox, const int *active, int step, const PcgS
                                                const double *, int);                              \
     template cudaError_t launch_bottom<T>(const BoxSet<T> &, const int *, int, cudaStream_t);   \
     template cudaError_t launch_zero<T>(const BoxSet<T> &, const int *, cudaStream_t);          \
-    template cudaError_t launch_coarse_vcycle<T>(const CoarseJob<T> *, int, const int *, int, int, \
-                                                 cudaStream_t, int);                                \
+    template cudaError_t launch_coarse_vcycle<T>(const CoarseJob<T> *, int, int, size_t,            \
+                                                 const int *, int, int, cudaStream_t, int, bool);   \
     template cudaError_t launch_exchange<T>(const BoxSet<T> &, const int *, const ExchRec *, int,  \
                                             int, cudaStream_t, int);                                         \
     template cudaError_t launch_guard_fill<T>(const BoxSet<T> &, T, cudaStream_t);                 \

@@ -319,7 +319,8 @@ static int choose_zc(const std::vector<Box<T>> &boxes, long long slots, double *
     return best;
 }
 
-// Cell limit of the levels run by the one-CTA coarse kernel.
+// Levels of at most this many cells always run inside the coarse kernel;
+// their residuals are restricted from all eight children.
 template <class T>
 static long long coarse_limit(const mg_opts &o)
 {
@@ -327,6 +328,88 @@ static long long coarse_limit(const mg_opts &o)
     if (o.coarse_cells > 0) return o.coarse_cells;
     return sizeof(T) == sizeof(double) ? 1024 : 4096;
 }
+
+// Shared-memory plan of box b's coarse V-cycle from level lc on a cluster of
+// cl CTAs (the job's ndist, nzc, scratch and level offsets); returns the bytes
+// a CTA needs.
+template <class T>
+static size_t plan_tail_with(const Solver *s, int b, int lc, int cl, bool split_d, CoarseJob<T> *J)
+{
+    const int nl = s->nlev[b];
+    const long long lim = coarse_limit<T>(s->opts);
+    auto cells = [&](int l) {
+        const auto &d = s->dims[b][l];
+        return (long long)d[0] * d[1] * d[2];
+    };
+    J->nlev = nl - lc;
+    J->box = b;
+    J->per = s->bc >> 6;
+    J->ndist = 0;
+    if (cl > 1)
+        while (lc + J->ndist < nl - 1 && cells(lc + J->ndist) > kTailSolo) ++J->ndist;
+    const int nd = J->ndist;
+    J->nzc = nd > 0 ? s->dims[b][lc + nd - 1][2] : 1;
+    size_t used = 0;
+    long long scratch = 0;
+    auto take = [&](long long n) {
+        const size_t o = used;
+        used += (size_t)round_up(n, 16 / (long long)sizeof(T));
+        return (int)o;
+    };
+    for (int l = lc; l < nl; ++l) {
+        const auto &d = s->dims[b][l];
+        const long long nx = d[0], ny = d[1];
+        const long long np = l - lc < nd ? (long long)((J->nzc + cl - 1) / cl) << (nd - 1 - (l - lc))
+                                         : d[2];
+        TailLevel &L = J->tl[l - lc];
+        // rows of f, 1/D and D (the coarsest level's f in natural order)
+        L.hp = l < nl - 1 && sizeof(T) == sizeof(double) ? (int)round_up(nx / 2, 2) : 0;
+        const long long fp = L.hp ? 2 * L.hp : nx;
+        L.phi = take((np + 2) * (nx + 2) * (ny + 2));
+        L.f = take(np * ny * fp);
+        L.red = s->opts.nu1 > 0 && !s->opts.full_residual && cells(l) > lim;
+        if (l == nl - 1) break;
+        L.wx = take(np * ny * (nx + 2));
+        L.wy = take(np * (ny + 1) * nx);
+        L.wz = take((np + 1) * ny * nx);
+        L.inv = take(np * ny * fp);
+        L.dg = -1;
+        if (sizeof(T) == sizeof(double) && (l - lc >= nd || split_d)) L.dg = take(np * ny * fp);
+        // residuals: the first CTA gathers those of the last split level
+        const long long own = l - lc == nd - 1 ? cells(l) : np * ny * nx;
+        scratch = std::max(scratch, own / (L.red ? 2 : 1));
+    }
+    J->scratch = take(scratch);
+    // the coarsest inverse, when small
+    const long long nb = cells(nl - 1);
+    J->ainv = nb * nb <= 4096 ? take(nb * nb) : -1;
+    return used * sizeof(T);
+}
+
+// The split levels' D in shared memory too if that fits, else from global.
+template <class T>
+static size_t plan_tail(const Solver *s, int b, int lc, int cl, CoarseJob<T> *J)
+{
+    const size_t n = plan_tail_with(s, b, lc, cl, true, J);
+    return n <= (size_t)kTailSmem ? n : plan_tail_with(s, b, lc, cl, false, J);
+}
+
+// CTAs of the cluster that runs each box's coarse levels: 16 (the most the
+// hardware takes) as long as every box's cluster can be resident at once.
+template <class T>
+static int tail_cluster(int nbox)
+{
+    for (int cl = 16; cl > 1; cl /= 2)
+        if (tail_clusters<T>(cl, kTailSmem) >= nbox) return cl;
+    tail_clusters<T>(1, kTailSmem);
+    return 1;
+}
+
+// A level joins the cluster's part while a pass over it costs less there than
+// the launch it saves (about 3 us): its FP64 updates take 16 x 7 / 32 cycles
+// a pair of cells on one SM's narrow pipe, 1.7 us for 32^3 on 16 SMs; FP32
+// levels of that size cost their loads of the weights instead.
+static bool tail_worth(long long cells, int cl) { return cells <= 3400LL * cl; }
 
 // Tensor maps of every box of an FP32 level set (TMA sweep); false if the
 // driver cannot encode them.
@@ -371,26 +454,32 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
     std::vector<CoarseJob<T>> jobs;
     const long long lim = coarse_limit<T>(s->opts);
     H.lc.assign(s->nbox, 0);
+    H.tail_cl = lim > 0 && !s->cg_bottom && !s->coupled ? tail_cluster<T>(s->nbox) : 1;
+    H.tail_smem = 0;
     for (int b = 0; b < s->nbox; ++b) {
         fine.push_back(make_box(s, H, b, 0));
         bottom.push_back(make_box(s, H, b, s->nlev[b] - 1));
-        // first level small enough for the coarse kernel (the coarsest level
-        // always is: it is solved there when the kernel is off)
+        // first level of the coarse kernel (the coarsest level always is one:
+        // it is solved there when the kernel is off): every level within the
+        // limit, then finer ones (never the finest, whose cycle also judges
+        // convergence) as long as they pay and fit
         int lc = s->nlev[b] - 1;
-        if (lim > 0 && !s->cg_bottom) {
-            for (int l = 0; l < s->nlev[b]; ++l) {
-                const auto &d = s->dims[b][l];
-                if ((long long)d[0] * d[1] * d[2] <= lim && s->nlev[b] - l <= kMaxCoarse) {
-                    lc = l;
-                    break;
-                }
-            }
-        }
-        H.lc[b] = lc;
         CoarseJob<T> J;
         memset(&J, 0, sizeof J);
-        J.nlev = s->nlev[b] - lc;
-        J.box = b;
+        auto fits = [&](int l) {
+            return s->nlev[b] - l <= kMaxCoarse && plan_tail(s, b, l, H.tail_cl, &J) <= (size_t)kTailSmem;
+        };
+        if (lim > 0 && !s->cg_bottom) {
+            auto cells = [&](int l) {
+                const auto &d = s->dims[b][l];
+                return (long long)d[0] * d[1] * d[2];
+            };
+            while (lc > 0 && cells(lc - 1) <= lim && fits(lc - 1)) --lc;
+            if (s->opts.coarse_cells == 0)
+                while (lc > 1 && tail_worth(cells(lc - 1), H.tail_cl) && fits(lc - 1)) --lc;
+        }
+        H.lc[b] = lc;
+        H.tail_smem = std::max(H.tail_smem, plan_tail(s, b, lc, H.tail_cl, &J));
         for (int l = lc; l < s->nlev[b]; ++l) J.lv[l - lc] = make_box(s, H, b, l);
         jobs.push_back(J);
     }
@@ -436,6 +525,7 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
         plans.push_back(plan_set(blob, &H.smooth[l], set));
     }
     H.njobs = (int)jobs.size();
+    H.tail_zero = *std::min_element(H.lc.begin(), H.lc.end()) > 0;
     *jobs_off = blob.put(jobs.data(), jobs.size() * sizeof(CoarseJob<T>));
     if (s->cg_bottom) {
         const auto &db = s->dims[0][s->nlev[0] - 1];
@@ -974,19 +1064,6 @@ int solver_create(Solver **out, int nbox, const int (*n)[3], const double *dx, i
         }
         s->ichunk = s->ipart + np;
         s->icstart = reinterpret_cast<const int *>(s->desc + icst_at);
-    }
-    if (periodic) {
-        // the coarse jobs' exchange records, now that their address is known
-        auto link = [&](size_t at, int lc, auto *tag) {
-            using J = std::remove_pointer_t<decltype(tag)>;
-            J *job = reinterpret_cast<J *>(blob.bytes.data() + at);
-            for (int l = 0; l < job->nlev; ++l) {
-                job->rec[l] = reinterpret_cast<const ExchRec *>(s->desc + xrec_at[lc + l]);
-                job->nrec[l] = s->nxrec[lc + l];
-            }
-        };
-        link(jobs64, s->h64.lc[0], (CoarseJob<double> *)nullptr);
-        if (s->has32) link(jobs32, s->h32.lc[0], (CoarseJob<float> *)nullptr);
     }
     e = cudaMemcpy(s->desc, blob.bytes.data(), blob.bytes.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -1561,8 +1638,9 @@ static cudaError_t enqueue_vcycle(Solver *s, const Hier<T> &H, cudaStream_t st,
                              H.cggrid, sizeof(T) == sizeof(double) ? kCgTol64 : kCgTol32,
                              sizeof(T) == sizeof(double) ? kCgMaxIt64 : kCgMaxIt32, st);
     else
-        e = launch_coarse_vcycle(H.jobs, H.njobs, s->active, s->opts.nu1, s->opts.nu2, st,
-                                 sym ? 1 : 0);
+        // (a hierarchy that starts in the kernel starts from the iterate)
+        e = launch_coarse_vcycle(H.jobs, H.njobs, H.tail_cl, H.tail_smem, s->active, s->opts.nu1,
+                                 s->opts.nu2, st, sym ? 1 : 0, H.tail_zero);
     if (e != cudaSuccess) return e;
     for (int l = nl - 1; l >= 0; --l) {
         const BoxSet<T> &S = H.smooth[l];
