@@ -31,7 +31,7 @@ constexpr int kSweepThreads = kTX * kSweepWarps;
 // The fused sweep indexes a level with 32-bit offsets: levels of at least
 // this many elements smooth with single-colour passes instead.
 constexpr long long kSweepMaxElems = (1LL << 31) - 1;
-constexpr int kColZ = 16;     // planes per thread of the column kernels (norms)
+constexpr int kColZ = 16;     // most planes per thread of the column kernels (norms)
 
 inline __host__ __device__ long long round_up(long long v, long long m) { return (v + m - 1) / m * m; }
 // wide: the layout of the boxes of a coupled level, whose guard cells hold
@@ -65,6 +65,8 @@ struct Box {
     const T *ainv;   // coarsest level only: dense A^{-1}, row-major n x n
     T *phic;         // next-coarser level solution (zeroed by restriction)
     T *fc;           // next-coarser level right-hand side
+    const T *cinvD;  // next-coarser level 1/D if its first red pass is folded into the
+                     // restriction (phic is left as that pass makes it), else NULL
     int nx, ny, nz;
     int P;           // row pitch
     long long Q;     // plane pitch
@@ -72,6 +74,7 @@ struct Box {
     long long cQ;    // coarse plane pitch
     int box;         // index of the box in its batch
     int zc;          // planes per CTA of the fused sweep (chosen on the host)
+    int cd;          // planes per thread of the column kernels (0: kColZ; see col_depth)
     int par;         // colour of local cell (0,0,0): (sum of the box's lower corner) % 2 on a
                      // coupled level (red = global i+j+k even), else 0
     int rb;          // 1: f, invD and D are colour-split (see split_at); 0: natural layout
@@ -87,6 +90,13 @@ __host__ __device__ __forceinline__ long long split_at(int i, int j, int k, int 
                                                        long long Q)
 {
     return (long long)k * Q + (long long)j * P + (((i + j + k + par) & 1) ? (P >> 1) : 0) + (i >> 1);
+}
+
+// Planes per thread of the column kernels.
+template <class T>
+__host__ __device__ __forceinline__ int col_depth(const Box<T> &B)
+{
+    return B.cd ? B.cd : kColZ;
 }
 
 // Colour-split f / invD / D in use: only FP64 levels split (a compile-time
@@ -116,7 +126,7 @@ __host__ __device__ __forceinline__ long long fidx(const Box<T> &B, int i, int j
 // Index spaces that kernels tile: all cells, red-black pairs along x
 // (ceil(nx/2) per row), the cells of the next-coarser level, pairs along x
 // with z cut into chunks of kSweepZ planes (the fused sweep marches in z), or
-// cells with z cut into chunks of kColZ planes (one thread per column chunk).
+// cells with z cut into chunks of col_depth planes (one thread per column chunk).
 enum TileKind {
     TK_CELL = 0,
     TK_PAIR = 1,
@@ -125,21 +135,22 @@ enum TileKind {
     TK_COLZ = 4,
     TK_FACE = 5,   // positions [0, nx] x [0, ny] x [0, nz] (every stored face)
     TK_CFACE = 6,  // positions of the next-coarser level's faces
-    TK_PCOLZ = 7,  // red-black pairs along x, z in chunks of kColZ planes
+    TK_PCOLZ = 7,  // red-black pairs along x, z in chunks of col_depth planes
     TK_NKIND = 8
 };
 
-// zc: planes per CTA of the fused sweep (TK_SWEEP only).
+// zc: planes per CTA of the fused sweep (TK_SWEEP only); cd: planes per
+// column (TK_COLZ, TK_PCOLZ).
 inline __host__ __device__ void tile_extent(int kind, int nx, int ny, int nz, int &ex, int &ey,
-                                            int &ez, int zc = kSweepZ)
+                                            int &ez, int zc = kSweepZ, int cd = kColZ)
 {
     if (kind == TK_PAIR) { ex = (nx + 1) / 2; ey = ny; ez = nz; }
     else if (kind == TK_COARSE) { ex = nx / 2; ey = ny / 2; ez = nz / 2; }
     else if (kind == TK_SWEEP) { ex = (nx + 1) / 2; ey = ny; ez = (nz + zc - 1) / zc; }
-    else if (kind == TK_COLZ) { ex = nx; ey = ny; ez = (nz + kColZ - 1) / kColZ; }
+    else if (kind == TK_COLZ) { ex = nx; ey = ny; ez = (nz + cd - 1) / cd; }
     else if (kind == TK_FACE) { ex = nx + 1; ey = ny + 1; ez = nz + 1; }
     else if (kind == TK_CFACE) { ex = nx / 2 + 1; ey = ny / 2 + 1; ez = nz / 2 + 1; }
-    else if (kind == TK_PCOLZ) { ex = (nx + 1) / 2; ey = ny; ez = (nz + kColZ - 1) / kColZ; }
+    else if (kind == TK_PCOLZ) { ex = (nx + 1) / 2; ey = ny; ez = (nz + cd - 1) / cd; }
     else { ex = nx; ey = ny; ez = nz; }
 }
 
@@ -155,10 +166,11 @@ inline __host__ __device__ bool tile_flat(int kind, int ex)
     return kind != TK_SWEEP && kind != TK_FACE && kind != TK_CFACE && ex % kTX != 0;
 }
 
-inline __host__ __device__ int tiles_of(int kind, int nx, int ny, int nz, int zc = kSweepZ)
+inline __host__ __device__ int tiles_of(int kind, int nx, int ny, int nz, int zc = kSweepZ,
+                                        int cd = kColZ)
 {
     int ex, ey, ez;
-    tile_extent(kind, nx, ny, nz, ex, ey, ez, zc);
+    tile_extent(kind, nx, ny, nz, ex, ey, ez, zc, cd);
     const int ty = tile_rows(kind);
     if (tile_flat(kind, ex)) {
         const long long per = (long long)kTX * ty;
@@ -322,9 +334,28 @@ __device__ __forceinline__ TilePos tile_pos(int kind, int nx, int ny, int nz, in
 }
 
 // Fixed-order block sum of one double per thread (blockDim = kTX x kTY):
-// warp shuffles, then warp 0 adds the 8 warp sums in order.  Result valid in
-// thread (0, 0).
+// through shared memory, warp 0 adding 8 values a lane and then its lanes.  13
+// FP64 instructions a CTA on GB300's narrow FP64 pipe (a shuffle tree in every
+// warp takes 48), 8 of them dependent (~100 cycles each).  Result valid in
+// thread (0, 0).  A caller that sums again separates the calls by a barrier.
 __device__ __forceinline__ double block_sum(double v)
+{
+    __shared__ double part[kThreads];
+    const int tid = threadIdx.y * kTX + threadIdx.x;
+    part[tid] = v;
+    __syncthreads();
+    double s = 0.0;
+    if (tid < 32) {
+        const double *q = part + tid;
+        s = ((q[0] + q[32]) + (q[64] + q[96])) + ((q[128] + q[160]) + (q[192] + q[224]));
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    }
+    return s;
+}
+
+// The same sum in another fixed order: a shuffle tree in every warp, then the
+// 8 warps in turn.
+__device__ __forceinline__ double block_sum_ordered(double v)
 {
     __shared__ double warp_part[kThreads / 32];
     int tid = threadIdx.y * kTX + threadIdx.x;
@@ -334,6 +365,21 @@ __device__ __forceinline__ double block_sum(double v)
     double s = 0.0;
     if (tid == 0)
         for (int w = 0; w < kThreads / 32; ++w) s += warp_part[w];
+    return s;
+}
+
+// Sum of one double per thread of a 1024-thread CTA, fixed order (shuffle
+// trees); valid in thread 0.
+__device__ __forceinline__ double block_sum_1024(double s)
+{
+    __shared__ double wsum[32];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        s = wsum[threadIdx.x];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    }
     return s;
 }
 

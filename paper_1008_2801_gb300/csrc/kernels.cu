@@ -272,9 +272,9 @@ __global__ void __launch_bounds__(kThreads, 8) k_rbgs_pass_oop(BoxSet<T> S,
 }
 
 // The same pass with the residual norm: each thread takes its pair through a
-// column of kColZ planes (TK_PCOLZ tiles), so the block reduction of the
+// column of col_depth planes (TK_PCOLZ tiles), so the block reduction of the
 // partial sums (FP64 adds and shuffles, costly on GB300's narrow FP64 pipe)
-// is paid once per kColZ cells instead of once per cell.
+// is paid once per column instead of once per cell.
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_rbgs_pass_oop_norm(BoxSet<T> S,
                                                                     const int *__restrict__ active,
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(kThreads) k_rbgs_pass_oop_norm(BoxSet<T> S,
     TilePos p = tile_pos(TK_PCOLZ, B.nx, B.ny, B.nz, t - ts[b]);
     double r2 = 0.0;
     if (p.y < B.ny && 2 * p.x < B.nx) {
-        const int z0 = p.z * kColZ, z1 = min(z0 + kColZ, B.nz);
+        const int cz = col_depth(B), z0 = p.z * cz, z1 = min(z0 + cz, B.nz);
 #pragma unroll 1
         for (int k = z0; k < z1; ++k) oop_pair(B, color, from2, p.y, k, 2 * p.x, true, r2);
     }
@@ -500,8 +500,22 @@ k_rbgs_sweep(BoxSet<T> S, const int *__restrict__ active, int src_is_phi2)
 
 // ------------------------------------------- residual + restriction ----
 
+// The coarse right-hand side r of coarse cell (I, J, K) and the start of the
+// coarse solution: 0, or (cinvD given) the coarse level's first red pass from
+// 0 already applied: -r / D on its red cells (the value of the pass's FMA
+// chain, whose products are all zero), which saves that pass: one of eight a
+// cycle on every coarse level, 17 us on 128^3, 3 to 4 on the small ones.
+template <class T>
+__device__ __forceinline__ void put_coarse(const Box<T> &B, int I, int J, int K, T r)
+{
+    const long long cf = cfidx(B, I, J, K);
+    B.fc[cf] = r;
+    B.phic[(long long)K * B.cQ + (long long)J * B.cP + I] =
+        B.cinvD && !((I + J + K + B.cpar) & 1) ? -r * B.cinvD[cf] : T(0);
+}
+
 // One coarse cell per thread, one tile of TK_COARSE: fc = mean over the 8
-// children of f - A phi, phic = 0.
+// children of f - A phi, phic its start.
 template <class T, bool FC>
 __device__ __forceinline__ void restrict_tile(const BoxSet<T> &S, const int *__restrict__ active,
                                               int t)
@@ -532,9 +546,7 @@ __device__ __forceinline__ void restrict_tile(const BoxSet<T> &S, const int *__r
         return sum;
     };
     const T sum = B.D ? children(std::true_type{}) : children(std::false_type{});
-    const long long cc = (long long)K * B.cQ + (long long)J * B.cP + I;
-    B.fc[cfidx(B, I, J, K)] = sum * T(0.125);
-    B.phic[cc] = T(0);
+    put_coarse(B, I, J, K, sum * T(0.125));
 }
 
 template <class T, bool FC>
@@ -576,9 +588,7 @@ __device__ __forceinline__ T restrict_red_cell(const Box<T> &B, int I, int J, in
                                : red4(std::true_type{}, std::false_type{}))
                       : (B.par ? red4(std::false_type{}, std::true_type{})
                                : red4(std::false_type{}, std::false_type{}));
-    const long long cc = (long long)K * B.cQ + (long long)J * B.cP + I;
-    B.fc[cfidx(B, I, J, K)] = sum * T(0.125);
-    B.phic[cc] = T(0);
+    put_coarse(B, I, J, K, sum * T(0.125));
     return r2;
 }
 
@@ -685,7 +695,7 @@ __global__ void __launch_bounds__(kThreads) k_residual_field(BoxSet<T> S)
 
 // mode 0: residual of every cell; 1: f; 2: residual of the red cells only
 // (right after a red-black sweep), one thread per red-black pair so that no
-// lane idles.  Each thread adds a column of kColZ planes.
+// lane idles.  Each thread adds a column of col_depth planes.
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_norm_partials(BoxSet<T> S, const int *__restrict__ active,
                                                             int mode, double *__restrict__ partials)
@@ -702,7 +712,7 @@ __global__ void __launch_bounds__(kThreads) k_norm_partials(BoxSet<T> S, const i
     const int ex = mode == 2 ? (B.nx + 1) / 2 : B.nx;
     auto column = [&](auto has_d) {
         constexpr bool HD = decltype(has_d)::value;
-        const int z0 = p.z * kColZ, z1 = min(z0 + kColZ, B.nz);
+        const int cz = col_depth(B), z0 = p.z * cz, z1 = min(z0 + cz, B.nz);
         for (int k = z0; k < z1; ++k) {
             const int x = mode == 2 ? 2 * p.x + ((p.y + k + B.par) & 1) : p.x;
             if (x >= B.nx) continue;
@@ -737,7 +747,7 @@ __global__ void __launch_bounds__(kThreads) k_max_partials(BoxSet<double> S,
     const double *phi = (side && side[B.box]) ? B.phi2 : B.phi;
     double v = 0.0;
     if (p.x < B.nx && p.y < B.ny) {
-        const int z0 = p.z * kColZ, z1 = min(z0 + kColZ, B.nz);
+        const int cz = col_depth(B), z0 = p.z * cz, z1 = min(z0 + cz, B.nz);
         for (int k = z0; k < z1; ++k) {
             const long long c = (long long)k * B.Q + (long long)p.y * B.P + p.x;
             const long long cf = fidx(B, p.x, p.y, k);
@@ -781,7 +791,7 @@ __global__ void __launch_bounds__(1024) k_max_finish(BoxSet<double> S,
 }
 
 // One CTA of 1024 threads per box: thread q adds partials q, q + 1024, ...
-// in order, then a fixed shuffle tree and an ordered sum of the 32 warps.
+// in order, then fixed shuffle trees.
 template <class T>
 __global__ void __launch_bounds__(1024) k_norm_finish(BoxSet<T> S, const int *__restrict__ active,
                                                       const double *__restrict__ partials,
@@ -792,19 +802,14 @@ __global__ void __launch_bounds__(1024) k_norm_finish(BoxSet<T> S, const int *__
                                                       const int *__restrict__ ts)
 {
     pdl_wait();
-    __shared__ double wsum[32];
     const int b = blockIdx.x;
     const Box<T> &B = S.boxes[b];
     if (active && !active[B.box]) return;
     const int lo = ts[b], hi = ts[b + 1];
     double s = 0.0;
     for (int q = lo + (int)threadIdx.x; q < hi; q += 1024) s += partials[q];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = s;
-    __syncthreads();
+    const double tot = block_sum_1024(s);
     if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < 32; ++w) tot += wsum[w];
         const double nrm = mult ? sqrt(tot) * mult[B.box] : sqrt(tot);
         out[B.box] = nrm;
         if (copy) copy[B.box] = nrm;
@@ -1291,7 +1296,7 @@ __global__ void __launch_bounds__(kThreads) k_refine_residual(BoxSet<double> S64
     float acc = 0.f;
     if (p.x < B.nx && p.y < B.ny) {
         const float cri = (float)c_r_inv[B.box];
-        const int z0 = p.z * kColZ, z1 = min(z0 + kColZ, B.nz);
+        const int cz = col_depth(B), z0 = p.z * cz, z1 = min(z0 + cz, B.nz);
         auto column = [&](auto has_d) {
             constexpr bool HD = decltype(has_d)::value;
             for (int k = z0; k < z1; ++k) {
@@ -1366,8 +1371,8 @@ __global__ void __launch_bounds__(1024) k_judge(int nbox, const double *__restri
 // ------------------------------------------------- packing and helpers ----
 
 // The copies between the caller's packed arrays and the level layout, and
-// the zeroing of a level's phi, take one thread per cell column of kColZ
-// planes (TK_COLZ tiles): kColZ independent loads or stores in flight per
+// the zeroing of a level's phi, take one thread per cell column of col_depth
+// planes (TK_COLZ tiles): as many independent loads or stores in flight per
 // thread instead of one per one-plane CTA.  partials (f only, or NULL): also
 // the CTA's sum of f^2, as k_norm_partials in mode 1 forms it (the column's
 // FMAs in plane order, then block_sum), so that ||f|| needs no pass of its own.
@@ -1383,7 +1388,7 @@ __global__ void __launch_bounds__(kThreads) k_pack(BoxSet<double> S, const long 
     TilePos p = tile_pos(TK_COLZ, B.nx, B.ny, B.nz, t - ts[b]);
     double v = 0.0;
     if (p.x < B.nx && p.y < B.ny) {
-        const int z0 = p.z * kColZ, z1 = min(z0 + kColZ, B.nz);
+        const int cz = col_depth(B), z0 = p.z * cz, z1 = min(z0 + cz, B.nz);
         const long long us = (long long)B.ny * B.nx;
         const double *src = user + off[B.box] + ((long long)z0 * B.ny + p.y) * B.nx + p.x;
 #pragma unroll 4
@@ -1414,7 +1419,7 @@ __global__ void __launch_bounds__(kThreads) k_unpack(BoxSet<double> S, const lon
     const Box<double> &B = S.boxes[b];
     TilePos p = tile_pos(TK_COLZ, B.nx, B.ny, B.nz, t - ts[b]);
     if (p.x >= B.nx || p.y >= B.ny) return;
-    const int z0 = p.z * kColZ, z1 = min(z0 + kColZ, B.nz);
+    const int cz = col_depth(B), z0 = p.z * cz, z1 = min(z0 + cz, B.nz);
     const long long us = (long long)B.ny * B.nx;
     double *dst = user + off[B.box] + ((long long)z0 * B.ny + p.y) * B.nx + p.x;
     const double *src = ((side && side[B.box]) ? B.phi2 : B.phi) + (long long)z0 * B.Q +
@@ -1434,7 +1439,7 @@ __global__ void __launch_bounds__(kThreads) k_zero(BoxSet<T> S, const int *__res
     if (active && !active[B.box]) return;
     TilePos p = tile_pos(TK_COLZ, B.nx, B.ny, B.nz, t - ts[b]);
     if (p.x >= B.nx || p.y >= B.ny) return;
-    const int z0 = p.z * kColZ, z1 = min(z0 + kColZ, B.nz);
+    const int cz = col_depth(B), z0 = p.z * cz, z1 = min(z0 + cz, B.nz);
     T *dst = B.phi + (long long)z0 * B.Q + (long long)p.y * B.P + p.x;
 #pragma unroll 4
     for (int k = z0; k < z1; ++k, dst += B.Q) *dst = T(0);
@@ -2221,7 +2226,7 @@ __global__ void __launch_bounds__(kThreads) k_sum_partials(BoxSet<double> S, int
     TilePos p = tile_pos(TK_COLZ, B.nx, B.ny, B.nz, t - ts[b]);
     double v = 0.0;
     if (p.x < B.nx && p.y < B.ny) {
-        const int z0 = p.z * kColZ, z1 = min(z0 + kColZ, B.nz);
+        const int cz = col_depth(B), z0 = p.z * cz, z1 = min(z0 + cz, B.nz);
         for (int k = z0; k < z1; ++k)
             v += field ? B.phi[(long long)k * B.Q + (long long)p.y * B.P + p.x]
                        : B.f[fidx(B, p.x, p.y, k)];
@@ -2273,7 +2278,7 @@ __global__ void __launch_bounds__(kThreads) k_sub_mean(BoxSet<double> S, int fie
 // solution), p and q in two extra arrays.  Per-box scalars in PcgScalars.
 
 // PcgScalars (kernels.h): rz = <r, z> of the previous iteration (0 before the
-// first), rzn = <r, z> of this one, pq = <p, A p>, beta, alpha; [nbox] each.
+// first, then of this one), beta, alpha; [nbox] each.
 
 // A p at cell c (the operator; D stored on FP64 levels, element cf)
 __device__ __forceinline__ double apply_at(const double *__restrict__ p,
@@ -2291,14 +2296,21 @@ __device__ __forceinline__ double apply_at(const double *__restrict__ p,
 // op 1: p = z + beta p;
 // op 2: q = A p, partials of <p, q> (a launch of its own: A p reads the
 //       neighbours' p of op 1);
-// op 3: x += alpha p, r -= alpha q, partials of <r, r>, phi = 0 (the next
-//       V-cycle's zero start; z is dead once op 1 has used it);
+// op 3: x += alpha p, r -= alpha q, partials of <r, r>, phi = the next
+//       V-cycle's start (z is dead once op 1 has used it): 0 with the first
+//       red pass applied;
 // op 4 (start): x = phi (the initial guess), r = f - A x, p = 0, partials
 //       of <r, r>;
-// op 5: phi = x (before a restart from the true residual).
-// Partials per TK_COLZ tile (a thread per column of kColZ planes).
+// op 5: phi = x (before a restart from the true residual);
+// op 6: phi = the V-cycle's start (as op 3).
+// The op is a template argument: a run-time one was tested for every cell.
+// Partials per TK_COLZ tile (a thread per column of kColZ planes, whatever the
+// size, and block_sum_ordered: on high-contrast coefficients CG turns a
+// rounding of its dot products into a solution that differs by more than its
+// error at the usual tolerances, so their order stays what it was).
+template <int op>
 __global__ void __launch_bounds__(kThreads) k_pcg(BoxSet<double> S, const int *__restrict__ active,
-                                                  int op, double *const *__restrict__ pv,
+                                                  double *const *__restrict__ pv,
                                                   double *const *__restrict__ qv, PcgScalars sc,
                                                   double *__restrict__ partials)
 {
@@ -2312,45 +2324,82 @@ __global__ void __launch_bounds__(kThreads) k_pcg(BoxSet<double> S, const int *_
     double *P = pv[B.box], *Qa = qv[B.box];
     double v = 0.0;
     if (p.x < B.nx && p.y < B.ny) {
-        const int z0 = p.z * kColZ, z1 = min(z0 + kColZ, B.nz);
+        const int cz = col_depth(B), z0 = p.z * cz, z1 = min(z0 + cz, B.nz);
         const double be = op == 1 ? sc.beta[B.box] : 0.0, al = op == 3 ? sc.alpha[B.box] : 0.0;
-        for (int k = z0; k < z1; ++k) {
-            const long long c = (long long)k * B.Q + (long long)p.y * B.P + p.x;
-            const long long cf = fidx(B, p.x, p.y, k);
-            if (op == 0) {
-                v = fma(B.f[cf], B.phi[c], v);
-            } else if (op == 1) {
-                P[c] = fma(be, P[c], B.phi[c]);
-            } else if (op == 2) {
-                const double q = apply_at(P, B, c, cf);
-                Qa[c] = q;
-                v = fma(P[c], q, v);
-            } else if (op == 3) {
-                B.phi2[c] = fma(al, P[c], B.phi2[c]);
-                const double r = fma(-al, Qa[c], B.f[cf]);
-                B.f[cf] = r;
-                B.phi[c] = 0.0;
-                v = fma(r, r, v);
-            } else if (op == 4) {
-                B.phi2[c] = B.phi[c];
-                const double r = residual_at<double, true>(B.phi, B.f, B.wx, B.wy, B.wz, B.D, c,
-                                                           cf, B.P, B.Q);
-                B.f[cf] = r;
-                P[c] = 0.0;
-                v = fma(r, r, v);
-            } else {
-                B.phi[c] = B.phi2[c];
+        // the V-cycle's zero start with its first red pass applied (put_coarse)
+        auto start = [&](int i, int j, int k, double r, long long cf) {
+            return ((i + j + k + B.par) & 1) ? 0.0 : -r * B.invD[cf];
+        };
+        // a few planes' loads in flight before the first of their stores
+        constexpr int N = op == 2 || op == 4 ? 2 : 4;
+        for (int k0 = z0; k0 < z1; k0 += N) {
+            double x0[N], x1[N], x2[N];
+#pragma unroll
+            for (int u = 0; u < N; ++u) {
+                const int k = k0 + u;
+                if (k >= z1) break;
+                const long long c = (long long)k * B.Q + (long long)p.y * B.P + p.x;
+                const long long cf = fidx(B, p.x, p.y, k);
+                if (op == 0) {
+                    x0[u] = B.f[cf];
+                    x1[u] = B.phi[c];
+                } else if (op == 1) {
+                    x0[u] = P[c];
+                    x1[u] = B.phi[c];
+                } else if (op == 2) {
+                    x0[u] = apply_at(P, B, c, cf);
+                    x1[u] = P[c];
+                } else if (op == 3) {
+                    x0[u] = fma(al, P[c], B.phi2[c]);
+                    x1[u] = fma(-al, Qa[c], B.f[cf]);
+                    x2[u] = start(p.x, p.y, k, x1[u], cf);
+                } else if (op == 4) {
+                    x0[u] = B.phi[c];
+                    x1[u] = residual_at<double, true>(B.phi, B.f, B.wx, B.wy, B.wz, B.D, c, cf,
+                                                      B.P, B.Q);
+                } else if (op == 5) {
+                    x0[u] = B.phi2[c];
+                } else {
+                    x0[u] = start(p.x, p.y, k, B.f[cf], cf);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < N; ++u) {
+                const int k = k0 + u;
+                if (k >= z1) break;
+                const long long c = (long long)k * B.Q + (long long)p.y * B.P + p.x;
+                const long long cf = fidx(B, p.x, p.y, k);
+                if (op == 0) {
+                    v = fma(x0[u], x1[u], v);
+                } else if (op == 1) {
+                    P[c] = fma(be, x0[u], x1[u]);
+                } else if (op == 2) {
+                    Qa[c] = x0[u];
+                    v = fma(x1[u], x0[u], v);
+                } else if (op == 3) {
+                    B.phi2[c] = x0[u];
+                    B.f[cf] = x1[u];
+                    B.phi[c] = x2[u];
+                    v = fma(x1[u], x1[u], v);
+                } else if (op == 4) {
+                    B.phi2[c] = x0[u];
+                    B.f[cf] = x1[u];
+                    P[c] = 0.0;
+                    v = fma(x1[u], x1[u], v);
+                } else {
+                    B.phi[c] = x0[u];
+                }
             }
         }
     }
-    if (op != 1 && op != 5) {
-        const double sum = block_sum(v);
+    if (op != 1 && op < 5) {
+        const double sum = block_sum_ordered(v);
         if (threadIdx.x == 0 && threadIdx.y == 0) partials[t] = sum;
     }
 }
 
 // Mixed-precision preconditioner (the FP32 V-cycle applied to the FP64 r):
-// op 0: the FP32 right-hand side r / ||r|| and a zero FP32 start;
+// op 0: the FP32 right-hand side r / ||r|| and the FP32 cycle's start;
 // op 1: z = ||r|| e, the FP32 solution scaled back into the FP64 phi.
 // nrm: ||r|| per box (the last CG update's, or the start's).
 __global__ void __launch_bounds__(kThreads) k_pcg_mixed(BoxSet<double> S64, BoxSet<float> S32,
@@ -2369,51 +2418,47 @@ __global__ void __launch_bounds__(kThreads) k_pcg_mixed(BoxSet<double> S64, BoxS
     const long long c = (long long)p.z * B.Q + (long long)p.y * B.P + p.x;
     const double s = nrm[B.box];
     if (op == 0) {
-        E.f[c] = s > 0.0 ? (float)(B.f[fidx(B, p.x, p.y, p.z)] / s) : 0.0f;
-        E.phi[c] = 0.0f;
+        const float r = s > 0.0 ? (float)(B.f[fidx(B, p.x, p.y, p.z)] / s) : 0.0f;
+        E.f[c] = r;
+        // (the zero start with its first red pass applied, as in k_pcg)
+        E.phi[c] = ((p.x + p.y + p.z + E.par) & 1) ? 0.0f : -r * E.invD[c];
     } else {
         B.phi[c] = s * (double)E.phi[c];
     }
 }
 
-// Per-box scalars from finished sums.  step 0: rzn done -> beta = rzn / rz
-// (0 on the first iteration), rz = rzn;  step 1: pq done -> alpha = rz / pq.
-__global__ void k_pcg_scalars(int nbox, const int *__restrict__ active, int step, PcgScalars sc)
-{
-    pdl_wait();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nbox || (active && !active[b])) return;
-    if (step == 0) {
-        const double rz = sc.rz[b], rzn = sc.rzn[b];
-        sc.beta[b] = rz != 0.0 ? rzn / rz : 0.0;
-        sc.rz[b] = rzn;
-    } else {
-        const double pq = sc.pq[b];
-        sc.alpha[b] = pq != 0.0 ? sc.rz[b] / pq : 0.0;
-    }
-}
-
-// One CTA per box: out[box] = sum of the box's partials (fixed order), or
-// its square root.
-__global__ void __launch_bounds__(1024) k_sum_finish(BoxSet<double> S, const int *__restrict__ active,
+// One CTA per box: the sum of the box's partials (fixed order) and what the
+// iteration takes from it.  op 0: <r, z>, so beta = it / rz (0 on the first
+// iteration) and rz = it; op 2: <p, q>, alpha = rz / it; op 3, 4: out = its
+// square root.
+template <int op>
+__global__ void __launch_bounds__(1024) k_pcg_finish(BoxSet<double> S, const int *__restrict__ active,
                                                      const double *__restrict__ partials,
-                                                     double *__restrict__ out, int root)
+                                                     PcgScalars sc, double *__restrict__ out)
 {
     pdl_wait();
-    __shared__ double wsum[32];
     const int b = blockIdx.x;
-    const Box<double> &B = S.boxes[b];
-    if (active && !active[B.box]) return;
+    const int box = S.boxes[b].box;
+    if (active && !active[box]) return;
     const int *ts = S.tstart[TK_COLZ];
     double s = 0.0;
     for (int q = ts[b] + (int)threadIdx.x; q < ts[b + 1]; q += 1024) s += partials[q];
+    // (the order of the sums is fixed for good: see block_sum_ordered)
+    __shared__ double wsum[32];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int w = 0; w < 32; ++w) tot += wsum[w];
-        out[B.box] = root ? sqrt(tot) : tot;
+    if (threadIdx.x != 0) return;
+    double tot = 0.0;
+    for (int w = 0; w < 32; ++w) tot += wsum[w];
+    if (op == 0) {
+        const double rz = sc.rz[box];
+        sc.beta[box] = rz != 0.0 ? tot / rz : 0.0;
+        sc.rz[box] = tot;
+    } else if (op == 2) {
+        sc.alpha[box] = tot != 0.0 ? sc.rz[box] / tot : 0.0;
+    } else {
+        out[box] = sqrt(tot);
     }
 }
 
@@ -2807,6 +2852,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_level_down(BoxSet<T> S, const i
     }
     for (int sw = 0; sw < sweeps; ++sw)
         for (int color = 0; color < 2; ++color) {
+            if (op.red_done && sw == 0 && color == 0) continue;
             if (!exchange(0)) return;
             each(npair, [&](int t) { pass_tile(S, active, color, t); });
             if (!grid_sync(g)) return;
@@ -3522,15 +3568,26 @@ cudaError_t launch_norm_combine(int nbox, double *norm, cudaStream_t st)
 
 cudaError_t launch_pcg(const BoxSet<double> &S, const int *active, int op, double *const *pv,
                        double *const *qv, const PcgScalars &sc, double *partials,
-                       double *sum_out, cudaStream_t st)
+                       double *norm_out, cudaStream_t st)
 {
     if (S.ntiles[TK_COLZ] == 0) return cudaSuccess;
-    cudaError_t e =
-        pdl_launch(k_pcg, dim3(S.ntiles[TK_COLZ]), block2d(), 0, st, S, active, op, pv, qv, sc,
-                   partials);
-    if (e != cudaSuccess || op == 1 || op == 5 || !sum_out) return e;
-    return pdl_launch(k_sum_finish, dim3(S.nbox), dim3(1024), 0, st, S, active, partials, sum_out,
-                      op >= 3);
+    auto go = [&](auto tag) {
+        constexpr int OP = decltype(tag)::value;
+        cudaError_t e = pdl_launch(k_pcg<OP>, dim3(S.ntiles[TK_COLZ]), block2d(), 0, st, S, active,
+                                   pv, qv, sc, partials);
+        if (e != cudaSuccess || OP == 1 || OP >= 5) return e;
+        return pdl_launch(k_pcg_finish<OP>, dim3(S.nbox), dim3(1024), 0, st, S, active, partials,
+                          sc, norm_out);
+    };
+    switch (op) {
+    case 0: return go(std::integral_constant<int, 0>{});
+    case 1: return go(std::integral_constant<int, 1>{});
+    case 2: return go(std::integral_constant<int, 2>{});
+    case 3: return go(std::integral_constant<int, 3>{});
+    case 4: return go(std::integral_constant<int, 4>{});
+    case 5: return go(std::integral_constant<int, 5>{});
+    default: return go(std::integral_constant<int, 6>{});
+    }
 }
 
 cudaError_t launch_max_norm(const BoxSet<double> &S, const int *side, int field,
@@ -3550,13 +3607,6 @@ cudaError_t launch_pcg_mixed(const BoxSet<double> &S64, const BoxSet<float> &S32
     if (S64.ntiles[TK_CELL] == 0) return cudaSuccess;
     return pdl_launch(k_pcg_mixed, dim3(S64.ntiles[TK_CELL]), block2d(), 0, st, S64, S32, active,
                       op, nrm);
-}
-
-cudaError_t launch_pcg_scalars(int nbox, const int *active, int step, const PcgScalars &sc,
-                               cudaStream_t st)
-{
-    return pdl_launch(k_pcg_scalars, dim3((nbox + 127) / 128), dim3(128), 0, st, nbox, active,
-                      step, sc);
 }
 
 #define MG_INSTANTIATE(T)                                                                        \

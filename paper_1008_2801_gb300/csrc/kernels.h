@@ -167,6 +167,7 @@ struct LevelOps {
     int nu;              // sweeps (each a red and a black pass)
     int head_done;       // down, finest level after the look-ahead red pass (phi -> phi2): the
                          // first sweep ends with the black pass phi2 -> phi
+    int red_done;        // down: the first sweep's red pass is done (folded into what filled phi)
     int red;             // down: restrict the residual of the red children only
     int reverse;         // up: black before red in each sweep (symmetric cycle)
     const ExchRec *rec;  // ghost exchange before every pass and the residual (nrec = 0: none)
@@ -287,15 +288,15 @@ cudaError_t launch_norm_combine(int nbox, double *norm, cudaStream_t st);
 
 // ---- preconditioned CG (level-0 FP64 arrays; see kernels.cu) -------------
 struct PcgScalars {
-    double *rz, *rzn, *pq, *beta, *alpha;  // [nbox] each
+    double *rz, *beta, *alpha;  // [nbox] each
 };
-// op 0: <r, z> -> sum_out; 1: p = z + beta p; 2: q = A p and <p, q> -> sum_out;
-// 3: x += alpha p, r -= alpha q, phi = 0 and ||r|| -> sum_out;
-// 4: x = phi, r = f - A x, p = 0 and ||r|| -> sum_out (nullable); 5: phi = x.
+// op 0: rz = <r, z>, beta = rz / the previous rz (0 first); 1: p = z + beta p;
+// 2: q = A p, alpha = rz / <p, q>; 3: x += alpha p, r -= alpha q, phi = the next
+// cycle's start (0 with its first red pass applied) and ||r|| -> norm_out; 4: x = phi, r = f - A x, p = 0 and ||r|| -> norm_out;
+// 5: phi = x; 6: phi = the cycle's start.  partials: scratch of ops 0, 2, 3 and 4.
 cudaError_t launch_pcg(const BoxSet<double> &S, const int *active, int op, double *const *pv,
                        double *const *qv, const PcgScalars &sc, double *partials,
-                       double *sum_out, cudaStream_t st);
-// step 0: beta = rzn / rz (0 first), rz = rzn; step 1: alpha = rz / pq.
+                       double *norm_out, cudaStream_t st);
 // out[box] = max |f| (field 0) or max |f - A phi| (field 1; phi2 where
 // side[box] is set) over the box's level-0 cells.
 cudaError_t launch_max_norm(const BoxSet<double> &S, const int *side, int field,
@@ -304,7 +305,5 @@ cudaError_t launch_max_norm(const BoxSet<double> &S, const int *side, int field,
 // nrm * FP32 phi (the preconditioned residual z).
 cudaError_t launch_pcg_mixed(const BoxSet<double> &S64, const BoxSet<float> &S32, const int *active,
                              int op, const double *nrm, cudaStream_t st);
-cudaError_t launch_pcg_scalars(int nbox, const int *active, int step, const PcgScalars &sc,
-                               cudaStream_t st);
 
 }  // namespace mg

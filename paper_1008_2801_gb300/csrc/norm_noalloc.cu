@@ -80,7 +80,7 @@ __device__ __forceinline__ T resid(const Box<T> &B, long long c)
     return B.f[c] - fma(-D, B.phi[c], s);
 }
 
-// One CTA per column tile (32 x 8 columns, 16 planes): fixed-order sum of r^2.
+// One CTA per column tile (32 x 8 columns, col_depth planes): fixed-order sum of r^2.
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_noalloc_partials(Box<T> B, double *__restrict__ part)
 {
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kThreads) k_noalloc_partials(Box<T> B, double 
     const TilePos p = tile_pos(TK_COLZ, B.nx, B.ny, B.nz, t);
     double v = 0.0;
     if (p.x < B.nx && p.y < B.ny) {
-        const int z0 = p.z * kColZ, z1 = min(z0 + kColZ, B.nz);
+        const int cz = col_depth(B), z0 = p.z * cz, z1 = min(z0 + cz, B.nz);
         for (int k = z0; k < z1; ++k) {
             const long long c = (long long)k * B.Q + (long long)p.y * B.P + p.x;
             const double r = (double)resid<T>(B, c);
@@ -102,17 +102,10 @@ __global__ void __launch_bounds__(kThreads) k_noalloc_partials(Box<T> B, double 
 __global__ void __launch_bounds__(1024) k_noalloc_finish(const double *__restrict__ part, int n,
                                                          double *__restrict__ out)
 {
-    __shared__ double w[32];
     double s = 0.0;
     for (int q = threadIdx.x; q < n; q += 1024) s += part[q];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int i = 0; i < 32; ++i) tot += w[i];
-        *out = sqrt(tot);
-    }
+    const double tot = block_sum_1024(s);
+    if (threadIdx.x == 0) *out = sqrt(tot);
 }
 
 template <class T>

@@ -252,6 +252,23 @@ struct SetPlan {
     size_t ts_off[TK_NKIND];
 };
 
+// Planes per thread of the column kernels over a set: deep columns pay the
+// block reduction less often, shallow ones leave enough CTAs in flight.  The
+// look-ahead pass took 18.2 us on a 64^3 level with 16 planes (32 CTAs) and
+// 7.0 with 4, 146 and 166 us on 8 x 128^3 (2048 CTAs), 162 and 165 us on
+// 256^3: 4 planes below one wave of 16-plane CTAs (pairs, 8 an SM).
+template <class T>
+static void set_col_depth(const Solver *s, std::vector<Box<T>> &boxes)
+{
+    long long tiles = 0;
+    for (const auto &B : boxes) tiles += tiles_of(TK_PCOLZ, B.nx, B.ny, B.nz);
+    // (CG's dot products keep their order: see k_pcg)
+    for (auto &B : boxes) B.cd = tiles < 8LL * s->sms && !s->pcg ? 4 : kColZ;
+}
+template <class T>
+static int cd_of(const Box<T> &B) { return col_depth(B); }
+static int cd_of(const SetupBox &) { return kColZ; }
+
 template <class D>
 static SetPlan<D> plan_set(DescBlob &blob, DescSet<D> *target, const std::vector<D> &boxes)
 {
@@ -264,7 +281,7 @@ static SetPlan<D> plan_set(DescBlob &blob, DescSet<D> *target, const std::vector
         std::vector<int> ts(boxes.size() + 1, 0);
         for (size_t i = 0; i < boxes.size(); ++i) {
             const int zc = boxes[i].zc > 0 ? boxes[i].zc : kSweepZ;
-            ts[i + 1] = ts[i] + tiles_of(k, boxes[i].nx, boxes[i].ny, boxes[i].nz, zc);
+            ts[i + 1] = ts[i] + tiles_of(k, boxes[i].nx, boxes[i].ny, boxes[i].nz, zc, cd_of(boxes[i]));
             int ex, ey, ez;
             tile_extent(k, boxes[i].nx, boxes[i].ny, boxes[i].nz, ex, ey, ez, zc);
             if (tile_flat(k, ex)) target->flat |= 1 << k;
@@ -483,15 +500,17 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
         for (int l = lc; l < s->nlev[b]; ++l) J.lv[l - lc] = make_box(s, H, b, l);
         jobs.push_back(J);
     }
+    set_col_depth(s, fine);
     plans.push_back(plan_set(blob, &H.fine, fine));
     plans.push_back(plan_set(blob, &H.bottom, bottom));
     H.fused.assign(H.smooth.size(), 0);
+    H.red_done.assign(H.smooth.size(), 0);
     H.maps.assign(H.smooth.size(), nullptr);
     H.prol.assign(H.smooth.size(), 0);
     const bool tma = sizeof(T) == sizeof(float) && s->tma;
     const long long slots =
         (long long)s->sms * (tma ? sweep_tma_ctas_per_sm() : sweep_ctas_per_sm<T>());
-    for (int l = 0; l + 1 < s->maxlev; ++l) {
+    for (int l = s->maxlev - 2; l >= 0; --l) {   // (a level's descriptors depend on the one below)
         std::vector<Box<T>> set;
         for (int b = 0; b < s->nbox; ++b)
             if (l < H.lc[b]) set.push_back(make_box(s, H, b, l));
@@ -522,6 +541,21 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
                 H.prol[l] = prol ? 1 : 0;
             }
         }
+        // the level below, where it smooths with passes, takes its first red
+        // pass from this level's restriction (sets of up to 32^3 cells keep a
+        // launch per stage: they are launched only where the cluster kernel is
+        // off or has no place, and the launch counts are read there)
+        long long below = 0;
+        for (const auto &B : set)
+            if (l + 1 < H.lc[B.box]) below += (long long)(B.nx / 2) * (B.ny / 2) * (B.nz / 2);
+        const bool fold = s->opts.nu1 > 0 && l + 2 < s->maxlev && !H.fused[l + 1] &&
+                          below > 32 * 32 * 32;
+        for (auto &B : set)
+            if (fold && l + 1 < H.lc[B.box]) {
+                B.cinvD = H.lv[B.box][l + 1].invD;
+                H.red_done[l + 1] = 1;
+            }
+        set_col_depth(s, set);
         plans.push_back(plan_set(blob, &H.smooth[l], set));
     }
     H.njobs = (int)jobs.size();
@@ -804,8 +838,6 @@ int solver_create(Solver **out, int nbox, const int (*n)[3], const double *dx, i
             }
         }
         s->sc.rz = bb.take<double>(nbox);
-        s->sc.rzn = bb.take<double>(nbox);
-        s->sc.pq = bb.take<double>(nbox);
         s->sc.beta = bb.take<double>(nbox);
         s->sc.alpha = bb.take<double>(nbox);
         s->pcg_p = bb.take<double *>(nbox);
@@ -1474,10 +1506,12 @@ static cudaError_t pass_launch(Solver *s, const BoxSet<T> &S, int color, cudaStr
 // reverse: black before red in each sweep (single-colour passes only).
 // prolong_first: the first sweep also applies the level's prolongation
 // (fused TMA sweeps whose maps hold the coarse phi, nu >= 2).
+// red_done: the first sweep's red pass is already in phi (passes only).
 template <class T>
 static cudaError_t smooth(Solver *s, const BoxSet<T> &S, int nu, bool fine, bool fused,
                           const SweepMaps *maps, cudaStream_t st, int lvl = 0,
-                          bool reverse = false, bool prolong_first = false)
+                          bool reverse = false, bool prolong_first = false,
+                          bool red_done = false)
 {
     // one timed stretch per group of back-to-back launches, so that the
     // event records between launches do not count in each launch's time
@@ -1498,9 +1532,9 @@ static cudaError_t smooth(Solver *s, const BoxSet<T> &S, int nu, bool fine, bool
         left -= left / 2 * 2;
     }
     if (left > 0) {
-        const int sl = fine ? prof_begin(s, MG_PROF_PASS, st, 2 * left) : -1;
-        for (; left > 0; --left) {
-            for (int color = 0; color < 2; ++color) {
+        const int sl = fine ? prof_begin(s, MG_PROF_PASS, st, 2 * left - (red_done ? 1 : 0)) : -1;
+        for (; left > 0; --left, red_done = false) {
+            for (int color = red_done ? 1 : 0; color < 2; ++color) {
                 if ((e = exch(s, S, lvl, st)) != cudaSuccess) return e;
                 if ((e = pass_launch(s, S, reverse ? 1 - color : color, st)) != cudaSuccess)
                     return e;
@@ -1543,12 +1577,14 @@ static cudaError_t inner_judge(Solver *, const BoxSet<double> &, cudaStream_t)
 
 template <class T>
 static cudaError_t level_launch(Solver *s, const Hier<T> &H, int l, bool up, int nu,
-                                bool head_done, bool sym, cudaStream_t st)
+                                bool head_done, bool sym, cudaStream_t st,
+                                bool red_done = false)
 {
     const BoxSet<T> &S = H.smooth[l];
     LevelOps op{};
     op.nu = nu;
     op.head_done = head_done ? 1 : 0;
+    op.red_done = red_done ? 1 : 0;
     op.red = (!up && s->opts.nu1 > 0 && !s->opts.full_residual) ? 1 : 0;
     op.reverse = sym ? 1 : 0;
     if (s->xmode && s->nxrec[l] > 0) {
@@ -1598,9 +1634,11 @@ static cudaError_t enqueue_vcycle(Solver *s, const Hier<T> &H, cudaStream_t st,
     for (int l = part == 2 ? 1 : 0; l < (part == 1 ? std::min(nl, 1) : nl); ++l) {
         const BoxSet<T> &S = H.smooth[l];
         if (S.nbox == 0) continue;
+        // (CG's updates leave the finest level's start with its red pass applied)
+        const bool red_done = l > 0 ? H.red_done[l] != 0 : s->pcg;
         if (level_persistent(s, H, l)) {
-            if ((e = level_launch(s, H, l, false, s->opts.nu1, l == 0 && head_done, false, st)) !=
-                cudaSuccess)
+            if ((e = level_launch(s, H, l, false, s->opts.nu1, l == 0 && head_done, false, st,
+                                  red_done)) != cudaSuccess)
                 return e;
             if (l == 0 && part == 0) coarse = prof_begin(s, MG_PROF_COARSE, st);
             continue;
@@ -1615,7 +1653,8 @@ static cudaError_t enqueue_vcycle(Solver *s, const Hier<T> &H, cudaStream_t st,
             prof_end(s, sl, st);
             --nu1;
         }
-        if ((e = smooth(s, S, nu1, l == 0, H.fused[l] != 0, H.maps[l], st, l)) != cudaSuccess)
+        if ((e = smooth(s, S, nu1, l == 0, H.fused[l] != 0, H.maps[l], st, l, false, false,
+                        red_done)) != cudaSuccess)
             return e;
         int sl = l == 0 ? prof_begin(s, MG_PROF_RESTRICT, st) : -1;
         if ((e = exch(s, S, l, st)) != cudaSuccess) return e;
@@ -1919,14 +1958,12 @@ static cudaError_t enqueue_pcg(Solver *s, cudaStream_t st)
     }
     const BoxSet<double> &F = s->h64.fine;
     const int sl = prof_begin(s, MG_PROF_KRYLOV, st);
-    if ((e = launch_pcg(F, s->active, 0, s->pcg_p, s->pcg_q, s->sc, s->partials, s->sc.rzn, st)) !=
+    if ((e = launch_pcg(F, s->active, 0, s->pcg_p, s->pcg_q, s->sc, s->partials, nullptr, st)) !=
             cudaSuccess ||
-        (e = launch_pcg_scalars(s->nbox, s->active, 0, s->sc, st)) != cudaSuccess ||
         (e = launch_pcg(F, s->active, 1, s->pcg_p, s->pcg_q, s->sc, nullptr, nullptr, st)) !=
             cudaSuccess ||
-        (e = launch_pcg(F, s->active, 2, s->pcg_p, s->pcg_q, s->sc, s->partials, s->sc.pq, st)) !=
+        (e = launch_pcg(F, s->active, 2, s->pcg_p, s->pcg_q, s->sc, s->partials, nullptr, st)) !=
             cudaSuccess ||
-        (e = launch_pcg_scalars(s->nbox, s->active, 1, s->sc, st)) != cudaSuccess ||
         (e = launch_pcg(F, s->active, 3, s->pcg_p, s->pcg_q, s->sc, s->partials, s->dnorm, st)) !=
             cudaSuccess)
         return e;
@@ -2233,7 +2270,8 @@ int solver_solve(Solver *s, const double *f, double *phi, double tol, mg_stats *
         if (any) {
             CK(launch_pcg(H.fine, nullptr, 4, s->pcg_p, s->pcg_q, s->sc, s->partials, s->dnorm,
                           stream));   // ||r0|| (the mixed preconditioner's first scale)
-            CK(launch_zero(H.fine, nullptr, stream));
+            CK(launch_pcg(H.fine, nullptr, 6, s->pcg_p, s->pcg_q, s->sc, nullptr, nullptr,
+                          stream));
             CK(cudaMemsetAsync(s->sc.rz, 0, sizeof(double) * nbox, stream));
             for (int b = 0; b < nbox; ++b) side[b] = 1;
         }
@@ -2299,7 +2337,8 @@ int solver_solve(Solver *s, const double *f, double *phi, double tol, mg_stats *
             }
             if (!any) break;
             CKS(upload_active(s, bs, stream));
-            CK(launch_zero(H.fine, s->active, stream));
+            CK(launch_pcg(H.fine, s->active, 6, s->pcg_p, s->pcg_q, s->sc, nullptr, nullptr,
+                          stream));
             CK(cudaMemsetAsync(s->sc.rz, 0, sizeof(double) * nbox, stream));
         }
     }

@@ -29,6 +29,8 @@ struct Hier {
     std::vector<T *> ainv;                      // [box] dense coarsest-level inverse
     std::vector<BoxSet<T>> smooth;              // [level]: boxes not yet at their bottom
     std::vector<char> fused;                    // [level]: smooth with fused sweeps
+    std::vector<char> red_done;                 // [level]: its first red pass is folded into the
+                                                //   restriction above (Box::cinvD)
     std::vector<const SweepMaps *> maps;        // [level]: TMA maps of the level's boxes (or null)
     std::vector<char> prol;                     // [level]: the maps hold the coarse phi (fused
                                                 //   prolongation in the first post-smoothing sweep)
