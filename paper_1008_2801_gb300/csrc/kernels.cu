@@ -2138,38 +2138,105 @@ __global__ void k_project_correct(int nx, int ny, int nz, int P, long long Q, do
         w[((long long)k * ny + j) * nx + i] -= wzf[q] * h * (ph(i, j, k) - ph(i, j, k - 1));
 }
 
-// dbeta += chain of dL/dbeta_face through the harmonic mean (see mg.h); a
-// Neumann wall face (bit w of bcm) has no coefficient and adds nothing.
-// Arrays are contiguous (nz, ny, nx).
-__global__ void k_beta_grad(int nx, int ny, int nz, double inv_h2, int bcm,
-                            const double *__restrict__ beta, const double *__restrict__ phi,
-                            const double *__restrict__ lam, double *__restrict__ dbeta)
+// dbeta += chain of dL/dbeta_face through the harmonic mean (see mg.h),
+// summed over nrhs right-hand sides (phi and lam: consecutive (nz, ny, nx)
+// arrays); a Neumann wall face (bit w of bcm) has no coefficient and adds
+// nothing.
+//
+// The face between cells c and o adds g 2 beta_o^2 / (beta_c + beta_o)^2 to c
+// and g 2 beta_c^2 / (beta_c + beta_o)^2 to o, g = sum over right-hand sides of
+// (lam_o - lam_c)(phi_o - phi_c) / h^2.  Bound by the FP64 pipe: 9 operations a
+// cell and right-hand side, so every face's sum and its 2 / (beta_c + beta_o)^2
+// (rcp64, no division) are formed once, by the thread of its lower cell, and
+// handed to the upper cell through shared memory (x, y) or a register (z).  A
+// CTA marches kGradZ planes; the tile's lower x and y faces are formed again by
+// one warp each, its first z faces by every thread.  8 x 128^3: 540 us; one
+// launch per right-hand side with six faces and FP64 divisions a cell took
+// 8 x 397 us.
+constexpr int kGradZ = 8;
+__global__ void __launch_bounds__(kThreads) k_beta_grad(int nx, int ny, int nz, int nrhs,
+                                                        double inv_h2, int bcm,
+                                                        const double *__restrict__ beta,
+                                                        const double *__restrict__ phi,
+                                                        const double *__restrict__ lam,
+                                                        double *__restrict__ dbeta)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    const int k = blockIdx.z;
-    if (i >= nx || j >= ny || k >= nz) return;
-    const long long sx = 1, sy = nx, sz = (long long)nx * ny;
-    const long long c = k * sz + j * sy + i;
-    const double bc = beta[c], pc = phi[c], lc = lam[c];
-    double acc = 0.0;
-    auto face = [&](bool inside, long long o, int w) {
-        if (inside) {
-            const double bo = beta[o];
-            const double g = (lam[o] - lc) * (phi[o] - pc) * inv_h2;
-            const double s = bc + bo;
-            acc += g * (2.0 * bo * bo / (s * s));
-        } else if (!((bcm >> w) & 1)) {
-            acc += 2.0 * lc * pc * inv_h2;
+    __shared__ double sx[2][kTY][kTX + 1], sy[2][kTY + 1][kTX];
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const int i0 = blockIdx.x * kTX, j0 = blockIdx.y * kTY;
+    const int i = i0 + tx, j = j0 + ty;
+    const int k0 = blockIdx.z * kGradZ, k1 = min(k0 + kGradZ, nz);
+    const long long sy1 = nx, sz1 = (long long)nx * ny, cells = sz1 * nz;
+    const double two = 2.0 * inv_h2;
+    // the face between cell c and the upper cell c + d
+    auto face = [&](long long c, long long d) {
+        double g = 0.0;
+        for (int r = 0; r < nrhs; ++r) {
+            const double *p = phi + r * cells + c, *l = lam + r * cells + c;
+            g = fma(l[d] - l[0], p[d] - p[0], g);
         }
+        const double q = rcp64(beta[c] + beta[c + d]);
+        return (two * g) * (q * q);
     };
-    face(i > 0, c - sx, 0);
-    face(i < nx - 1, c + sx, 1);
-    face(j > 0, c - sy, 2);
-    face(j < ny - 1, c + sy, 3);
-    face(k > 0, c - sz, 4);
-    face(k < nz - 1, c + sz, 5);
-    dbeta[c] += acc;
+    const bool in = i < nx && j < ny;
+    const long long col = (long long)j * nx + i;
+    double zlo = (in && k0 > 0) ? face((k0 - 1) * sz1 + col, sz1) : 0.0;
+    for (int k = k0; k < k1; ++k) {
+        const long long c = k * sz1 + col;
+        const int s = k & 1;
+        const bool ux = in && i + 1 < nx, uy = in && j + 1 < ny, uz = in && k + 1 < nz;
+        double fx = 0.0, fy = 0.0, fz = 0.0, wall = 0.0;
+        if (in) {   // the three upper faces, their differences shared over one read
+            double gx = 0.0, gy = 0.0, gz = 0.0;
+            const long long dx = ux ? 1 : 0, dy = uy ? sy1 : 0, dz = uz ? sz1 : 0;
+            const bool edge = i == 0 || !ux || j == 0 || !uy || k == 0 || !uz;
+            for (int r = 0; r < nrhs; ++r) {
+                const double *p = phi + r * cells + c, *l = lam + r * cells + c;
+                const double pc = p[0], lc = l[0];
+                gx = fma(l[dx] - lc, p[dx] - pc, gx);
+                gy = fma(l[dy] - lc, p[dy] - pc, gy);
+                gz = fma(l[dz] - lc, p[dz] - pc, gz);
+                if (edge) wall = fma(lc, pc, wall);
+            }
+            const double b = beta[c];
+            double q = rcp64(b + beta[c + dx]);
+            fx = (two * gx) * (q * q);
+            q = rcp64(b + beta[c + dy]);
+            fy = (two * gy) * (q * q);
+            q = rcp64(b + beta[c + dz]);
+            fz = (two * gz) * (q * q);
+        }
+        sx[s][ty][tx + 1] = fx;
+        sy[s][ty + 1][tx] = fy;
+        if (ty == 0 && tx < kTY) {   // the tile's lower x faces
+            const int jj = j0 + tx;
+            sx[s][tx][0] = (i0 > 0 && i0 < nx + 1 && jj < ny)
+                               ? face(k * sz1 + (long long)jj * nx + i0 - 1, 1) : 0.0;
+        }
+        if (ty == 1)                 // its lower y faces
+            sy[s][0][tx] = (j0 > 0 && i < nx)
+                               ? face(k * sz1 + (long long)(j0 - 1) * nx + i, sy1) : 0.0;
+        __syncthreads();             // (two buffers: the next plane writes the other one)
+        if (in) {
+            auto sq = [&](long long o) { const double b = beta[o]; return b * b; };
+            const double xlo = sx[s][ty][tx], ylo = sy[s][ty][tx];
+            double acc = 0.0;
+            int walls = 0;
+            auto one = [&](bool inside, int w, double f, long long o) {
+                if (inside) acc = fma(f, sq(o), acc);
+                else if (!((bcm >> w) & 1)) ++walls;
+            };
+            one(i > 0, 0, xlo, c - 1);
+            one(ux, 1, fx, c + 1);
+            one(j > 0, 2, ylo, c - sy1);
+            one(uy, 3, fy, c + sy1);
+            one(k > 0, 4, zlo, c - sz1);
+            one(uz, 5, fz, c + sz1);
+            if (walls) acc = fma((double)walls * two, wall, acc);
+            dbeta[c] += acc;
+        }
+        zlo = fz;
+    }
 }
 
 // ------------------------------------------------------ wall values ----
@@ -3402,11 +3469,12 @@ cudaError_t launch_project_correct(int nx, int ny, int nz, double h, const doubl
     return counted(cudaGetLastError());
 }
 
-cudaError_t launch_beta_grad(int nx, int ny, int nz, double inv_h2, int bcm, const double *beta,
-                             const double *phi, const double *lam, double *dbeta, cudaStream_t st)
+cudaError_t launch_beta_grad(int nx, int ny, int nz, int nrhs, double inv_h2, int bcm,
+                             const double *beta, const double *phi, const double *lam,
+                             double *dbeta, cudaStream_t st)
 {
-    k_beta_grad<<<grid3(nx, ny, nz), block2d(), 0, st>>>(nx, ny, nz, inv_h2, bcm, beta, phi, lam,
-                                                         dbeta);
+    k_beta_grad<<<grid3(nx, ny, (nz + kGradZ - 1) / kGradZ), block2d(), 0, st>>>(
+        nx, ny, nz, nrhs, inv_h2, bcm, beta, phi, lam, dbeta);
     return counted(cudaGetLastError());
 }
 

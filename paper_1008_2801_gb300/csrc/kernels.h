@@ -256,8 +256,11 @@ cudaError_t launch_project_correct(int nx, int ny, int nz, double h, const doubl
                                    double *u, double *v, double *w, cudaStream_t st,
                                    bool wide = false);
 
-cudaError_t launch_beta_grad(int nx, int ny, int nz, double inv_h2, int bcm, const double *beta,
-                             const double *phi, const double *lam, double *dbeta, cudaStream_t st);
+// dbeta += the beta gradient of nrhs right-hand sides of one box (phi, lam:
+// consecutive arrays).
+cudaError_t launch_beta_grad(int nx, int ny, int nz, int nrhs, double inv_h2, int bcm,
+                             const double *beta, const double *phi, const double *lam,
+                             double *dbeta, cudaStream_t st);
 // fout = f - lift of the packed wall values (level-0 FP64 weights, layout of mg.h).
 cudaError_t launch_bc_lift(int nx, int ny, int nz, double inv_h, int bcm, const double *wx,
                            const double *wy, const double *wz, const double *vals,

@@ -420,7 +420,7 @@ int mg_op_beta_grad(const int n[3], double h, int bc, const double *beta, const 
 {
     if (bad_dims(n) || !(h > 0.0) || bc < 0 || bc > 63 || !beta || !phi || !lambda || !dbeta)
         return set_error(MG_ERR_INVALID_ARG, "bad argument");
-    CKO(launch_beta_grad(n[0], n[1], n[2], 1.0 / (h * h), bc, beta, phi, lambda, dbeta,
+    CKO(launch_beta_grad(n[0], n[1], n[2], 1, 1.0 / (h * h), bc, beta, phi, lambda, dbeta,
                          (cudaStream_t)stream));
     return MG_OK;
 }

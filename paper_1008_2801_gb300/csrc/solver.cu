@@ -2533,20 +2533,20 @@ int solver_adjoint(Solver *s, int nrhs, const double *phi, const double *g, doub
         s->stage_clean = false;  // the gradient below still reads staging buffers
         if (rc != MG_OK && rc != MG_ERR_NOT_CONVERGED && rc != MG_ERR_DIVERGED) return rc;
         worst = worse(worst, rc);
-        // lambda sits in the level-0 phi arrays; phi of this right-hand side
-        CKS(ensure_stage(s));
-        CK(launch_unpack(s->h64.fine, s->doff, s->stage_b, s->dside, stream));
-        s->kernels += 1;
+        // lambda: the solve's output, or for host arrays the staging copy it
+        // was unpacked into; phi of this right-hand side
+        bool wrong = false;
+        const double *lam = is_device_ptr(dLdf + o, s->dev, &wrong) ? dLdf + o : s->stage_b;
         const double *pd = nullptr;
         bool pst = false;
         CKS(device_view(s, phi + o, 0, true, stream, &pd, &pst));
-        for (int b = 0; b < s->nbox; ++b) {
+        // shared weights: every box is a right-hand side of box 0's beta
+        for (int b = 0; b < (s->shared ? 1 : s->nbox); ++b) {
             const auto &d = s->n[b];
-            const long long ob = s->shared ? 0 : s->off[b];
             s->kernels += 1;
-            CK(launch_beta_grad(d[0], d[1], d[2], 1.0 / (s->dx[b] * s->dx[b]), s->bc,
-                                s->beta + ob, pd + s->off[b], s->stage_b + s->off[b], db + ob,
-                                stream));
+            CK(launch_beta_grad(d[0], d[1], d[2], s->shared ? s->nbox : 1,
+                                1.0 / (s->dx[b] * s->dx[b]), s->bc, s->beta + s->off[b],
+                                pd + s->off[b], lam + s->off[b], db + s->off[b], stream));
         }
     }
     if (dbst)

@@ -92,3 +92,25 @@ def test_functional_solve_is_differentiable(cuda_device):
         s.set_beta(beta.detach())
         want, _ = s.solve((2 * phi).detach(), tol=1e-12)
     assert torch.allclose(f.grad, want, rtol=1e-8, atol=1e-12 * want.abs().max().item())
+
+
+@pytest.mark.parametrize("shape", [(4, 8, 32), (8, 9, 13), (10, 16, 48), (16, 24, 40)])
+@pytest.mark.parametrize("nrhs", [2, 5])
+def test_beta_gradient_of_several_right_hand_sides(cuda_device, shape, nrhs):
+    # one launch over all of them against one launch each (whose assembly is
+    # checked against the oracle), at full and part-filled tiles of 32 x 8
+    # columns and 8 planes; the bar is that of the assembly's own test
+    from paper_1008_2801_gb300 import ops as K
+
+    rng = np.random.default_rng(61)
+    dx = 1.0 / shape[2]
+    beta = torch.from_numpy(rng.uniform(0.5, 2.0, shape)).to(cuda_device)
+    phi, g = (torch.from_numpy(rng.uniform(-1, 1, (nrhs, *shape))).to(cuda_device)
+              for _ in range(2))
+    with Solver(shape, dx, device=cuda_device) as s:
+        s.set_beta(beta)
+        lam, got = s.adjoint(phi, g)
+    want = torch.zeros_like(beta)
+    for r in range(nrhs):
+        K.beta_grad(beta, phi[r].contiguous(), lam[r].contiguous(), dx, want)
+    assert (got - want).abs().max() <= 1e-13 * want.abs().max()
