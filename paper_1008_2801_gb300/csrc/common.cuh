@@ -53,6 +53,20 @@ inline __host__ __device__ long long level_elems(int nx, int ny, int nz, bool wi
     return pitch_plane(nx, ny, wide) * (nz + 2);
 }
 
+// Where a boundary cell's value also belongs: the guard cells of a neighbouring
+// box (coupled level) or of the opposite face (periodic axis).  The cells of
+// one face with tangential coordinates a in [a0, a1), b in [b0, b1) ((j, k) on
+// an x face, (i, k) on a y face, (i, j) on a z face) go to dst[a sa + b sb].  A
+// box's table starts with one record for each face x-, x+, .. z+ (empty ranges
+// where there is none); a face's further records follow through next.
+template <class T>
+struct PushRec {
+    T *dst;
+    int a0, a1, b0, b1;
+    long long sa, sb;
+    long long next;   // index in the table, 0: the last one
+};
+
 // One box at one level, as the cycle kernels see it.
 template <class T>
 struct Box {
@@ -67,6 +81,7 @@ struct Box {
     T *fc;           // next-coarser level right-hand side
     const T *cinvD;  // next-coarser level 1/D if its first red pass is folded into the
                      // restriction (phic is left as that pass makes it), else NULL
+    const PushRec<T> *prec;     // ghost exchanges: the box's push table, else NULL
     int nx, ny, nz;
     int P;           // row pitch
     long long Q;     // plane pitch

@@ -13,7 +13,8 @@ long long launch_counter();
 
 // One red (0) or black (1) Gauss-Seidel pass in place on Box::phi.
 template <class T>
-cudaError_t launch_rbgs_pass(const BoxSet<T> &S, const int *active, int color, cudaStream_t st);
+cudaError_t launch_rbgs_pass(const BoxSet<T> &S, const int *active, int color, cudaStream_t st,
+                             bool push = false);
 // One colour out of place (from2: phi2 -> phi, else phi -> phi2); partials
 // (FP64, nullable): per TK_PCOLZ tile, the sum of the squared residuals of the
 // source at the updated cells (finish with launch_norm_finish mode 2).

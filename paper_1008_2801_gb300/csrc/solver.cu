@@ -226,10 +226,64 @@ static Box<T> make_box(const Solver *s, const Hier<T> &H, int b, int l)
         B.par = parity(l);
         if (l + 1 < s->nlev[b]) B.cpar = parity(l + 1);
     }
+    const auto &pt = sizeof(T) == sizeof(double) ? s->push64 : s->push32;
+    if (!pt.empty())
+        B.prec = reinterpret_cast<const PushRec<T> *>(s->pushmem + pt[(size_t)l * s->nbox + b]);
     // FP64 levels keep f, 1/D and D colour-split: a single-colour pass then
     // reads only its own colour's sectors of them
     B.rb = sizeof(T) == sizeof(double) ? 1 : 0;
     return B;
+}
+
+// Push tables of every box and level with ghost exchanges: the level's
+// exchange records by source box and face.
+template <class T>
+static void build_push(const Solver *s, const Hier<T> &H, std::vector<char> &bytes,
+                       std::vector<size_t> &off)
+{
+    for (int l = 0; l < s->maxlev; ++l)
+        for (int b = 0; b < s->nbox; ++b) {
+            std::vector<PushRec<T>> recs[6];
+            for (const ExchRec &r : s->recs[l]) {
+                if (r.src != b) continue;
+                const auto &d = s->dims[r.dst][l];
+                const long long P = pitch_row(d[0], s->wide);
+                const long long Q = pitch_plane(d[0], d[1], s->wide);
+                const int at[3] = {r.di, r.dj, r.dk}, from[3] = {r.si, r.sj, r.sk},
+                          ext[3] = {r.ex, r.ey, r.ez};
+                const long long str[3] = {1, P, Q};
+                for (int x = 0; x < 3; ++x) {
+                    if (at[x] != -1 && at[x] != d[x]) continue;
+                    // the guard layer below the destination copies this box's
+                    // upper face, and the other way round
+                    const int u = x == 0 ? 1 : 0, v = x == 2 ? 1 : 2;
+                    PushRec<T> p{};
+                    p.dst = H.lv[r.dst][l].phi + at[x] * str[x] + (at[u] - from[u]) * str[u] +
+                            (at[v] - from[v]) * str[v];
+                    p.a0 = from[u];
+                    p.a1 = from[u] + ext[u];
+                    p.b0 = from[v];
+                    p.b1 = from[v] + ext[v];
+                    p.sa = str[u];
+                    p.sb = str[v];
+                    recs[2 * x + (at[x] == -1 ? 1 : 0)].push_back(p);
+                    break;
+                }
+            }
+            std::vector<PushRec<T>> tab(6);   // a face's first record, then the others
+            for (int f = 0; f < 6; ++f)
+                for (size_t q = 0, last = f; q < recs[f].size(); ++q) {
+                    if (q > 0) {
+                        tab[last].next = (long long)tab.size();
+                        last = tab.size();
+                        tab.push_back({});
+                    }
+                    tab[last] = recs[f][q];
+                }
+            off.push_back(bytes.size());
+            bytes.insert(bytes.end(), reinterpret_cast<char *>(tab.data()),
+                         reinterpret_cast<char *>(tab.data() + tab.size()));
+        }
 }
 
 // Host image of the descriptor arena; sets are patched to device addresses
@@ -924,6 +978,45 @@ int solver_create(Solver **out, int nbox, const int (*n)[3], const double *dx, i
         s->J.stall_limit = o.krylov ? 0 : 5;
     }
 
+    // ghost exchange records of every level (the cached communication pattern)
+    if (s->xmode) {
+        for (int l = 0; l < s->maxlev; ++l) {
+            std::vector<ExchRec> recs;
+            if (periodic) {
+                Brick bl;
+                int period[3];
+                for (int q = 0; q < 3; ++q) {
+                    bl.lo[q] = 0;
+                    bl.n[q] = s->dims[0][l][q];
+                    period[q] = ((bc >> (6 + q)) & 1) ? bl.n[q] : 0;
+                }
+                recs = periodic_exchange(bl, period);
+            } else {
+                std::vector<Brick> bl(nbox);
+                for (int b = 0; b < nbox; ++b)
+                    for (int d = 0; d < 3; ++d) {
+                        bl[b].lo[d] = clos[b][l][d];
+                        bl[b].n[d] = cdims[b][l][d];
+                    }
+                recs = level_exchange(bl);
+            }
+            s->nxrec.push_back((int)recs.size());
+            s->xmax.push_back(max_record_cells(recs));
+            s->recs.push_back(recs);
+        }
+        std::vector<char> bytes;
+        build_push(s, s->h64, bytes, s->push64);
+        if (s->has32) build_push(s, s->h32, bytes, s->push32);
+        e = dev_malloc(s, reinterpret_cast<void **>(&s->pushmem), bytes.size());
+        if (e == cudaSuccess)
+            e = cudaMemcpy(s->pushmem, bytes.data(), bytes.size(), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) {
+            solver_destroy(s);
+            return set_error(e == cudaErrorMemoryAllocation ? MG_ERR_OOM : MG_ERR_CUDA,
+                             "push tables: %s", cudaGetErrorString(e));
+        }
+    }
+
     // launch-set descriptors (+ packed offsets and side flags)
     DescBlob blob;
     std::vector<SetPlan<Box<double>>> p64;
@@ -1021,44 +1114,16 @@ int solver_create(Solver **out, int nbox, const int (*n)[3], const double *dx, i
                                         packed_bottom_bytes(B.nx * B.ny * B.nz, B.inv64 != nullptr));
         psu.push_back(plan_set(blob, &s->setup_bottom, bot));
     }
-    // coupled level: ghost exchange records of every level (the cached
-    // communication pattern) and the union numbering of the coarsest cells
+    // ghost exchange records of every level and the union numbering of the
+    // coarsest cells
     std::vector<size_t> xrec_at;
     size_t uoff_at = 0;
-    if (periodic) {
-        for (int l = 0; l < s->nlev[0]; ++l) {
-            const auto &d = s->dims[0][l];
-            Brick bl;
-            int period[3];
-            for (int q = 0; q < 3; ++q) {
-                bl.lo[q] = 0;
-                bl.n[q] = d[q];
-                period[q] = ((bc >> (6 + q)) & 1) ? d[q] : 0;
-            }
-            const std::vector<ExchRec> recs = periodic_exchange(bl, period);
-            s->nxrec.push_back((int)recs.size());
-            s->xmax.push_back(max_record_cells(recs));
+    if (s->xmode) {
+        for (const auto &recs : s->recs)
             xrec_at.push_back(blob.put(recs.data(), recs.size() * sizeof(ExchRec)));
-        }
-        std::vector<int> uo = {0, s->ub.n};
-        uoff_at = blob.put(uo.data(), uo.size() * sizeof(int));
-    }
-    if (coupled) {
-        for (int l = 0; l < clev; ++l) {
-            std::vector<Brick> bl(nbox);
-            for (int b = 0; b < nbox; ++b)
-                for (int d = 0; d < 3; ++d) {
-                    bl[b].lo[d] = clos[b][l][d];
-                    bl[b].n[d] = cdims[b][l][d];
-                }
-            const std::vector<ExchRec> recs = level_exchange(bl);
-            s->nxrec.push_back((int)recs.size());
-            s->xmax.push_back(max_record_cells(recs));
-            xrec_at.push_back(blob.put(recs.data(), recs.size() * sizeof(ExchRec)));
-        }
         std::vector<int> uo(nbox + 1, 0);
         for (int b = 0; b < nbox; ++b) {
-            const auto &d = cdims[b][clev - 1];
+            const auto &d = s->dims[b].back();
             uo[b + 1] = uo[b] + d[0] * d[1] * d[2];
         }
         uoff_at = blob.put(uo.data(), uo.size() * sizeof(int));
@@ -1169,6 +1234,7 @@ void solver_destroy(Solver *s)
     if (s->hjblock) cudaFreeHost(s->hjblock);
     dev_free(s, s->arena);
     dev_free(s, s->desc);
+    dev_free(s, s->pushmem);
     dev_free(s, s->ipart);
     dev_free(s, s->stage_a);
     if (s->hnorm) cudaFreeHost(s->hnorm);
@@ -1500,18 +1566,20 @@ template <class T>
 static cudaError_t pass_launch(Solver *s, const BoxSet<T> &S, int color, cudaStream_t st)
 {
     if (rhs_shared_level(s, S)) return launch_rbgs_pass_multi(S, s->active, color, 0, 0, st);
-    return launch_rbgs_pass(S, s->active, color, st);
+    return launch_rbgs_pass(S, s->active, color, st, s->xmode);
 }
 
 // reverse: black before red in each sweep (single-colour passes only).
 // prolong_first: the first sweep also applies the level's prolongation
 // (fused TMA sweeps whose maps hold the coarse phi, nu >= 2).
 // red_done: the first sweep's red pass is already in phi (passes only).
+// *fresh (in and out): the guard cells hold the neighbours' values (ghost
+// exchanges; a pass keeps them so).
 template <class T>
 static cudaError_t smooth(Solver *s, const BoxSet<T> &S, int nu, bool fine, bool fused,
                           const SweepMaps *maps, cudaStream_t st, int lvl = 0,
                           bool reverse = false, bool prolong_first = false,
-                          bool red_done = false)
+                          bool red_done = false, bool *fresh = nullptr)
 {
     // one timed stretch per group of back-to-back launches, so that the
     // event records between launches do not count in each launch's time
@@ -1535,7 +1603,8 @@ static cudaError_t smooth(Solver *s, const BoxSet<T> &S, int nu, bool fine, bool
         const int sl = fine ? prof_begin(s, MG_PROF_PASS, st, 2 * left - (red_done ? 1 : 0)) : -1;
         for (; left > 0; --left, red_done = false) {
             for (int color = red_done ? 1 : 0; color < 2; ++color) {
-                if ((e = exch(s, S, lvl, st)) != cudaSuccess) return e;
+                if (!(fresh && *fresh) && (e = exch(s, S, lvl, st)) != cudaSuccess) return e;
+                if (fresh) *fresh = true;
                 if ((e = pass_launch(s, S, reverse ? 1 - color : color, st)) != cudaSuccess)
                     return e;
             }
@@ -1653,11 +1722,12 @@ static cudaError_t enqueue_vcycle(Solver *s, const Hier<T> &H, cudaStream_t st,
             prof_end(s, sl, st);
             --nu1;
         }
+        bool fresh = false;   // guard cells: the restriction above or the copy in left them behind
         if ((e = smooth(s, S, nu1, l == 0, H.fused[l] != 0, H.maps[l], st, l, false, false,
-                        red_done)) != cudaSuccess)
+                        red_done, &fresh)) != cudaSuccess)
             return e;
         int sl = l == 0 ? prof_begin(s, MG_PROF_RESTRICT, st) : -1;
-        if ((e = exch(s, S, l, st)) != cudaSuccess) return e;
+        if (!fresh && (e = exch(s, S, l, st)) != cudaSuccess) return e;
         const bool red = s->opts.nu1 > 0 && !s->opts.full_residual;
         double *ip = red ? inner_partials(s, H, l) : nullptr;
         e = red ? launch_resid_restrict_red(S, s->active, st, ip)
@@ -1701,8 +1771,9 @@ static cudaError_t enqueue_vcycle(Solver *s, const Hier<T> &H, cudaStream_t st,
             if ((e = launch_prolong(S, s->active, st)) != cudaSuccess) return e;
             prof_end(s, sl, st);
         }
+        bool fresh = false;   // the prolongation changed the cells behind the guards
         if ((e = smooth(s, S, s->opts.nu2, l == 0, H.fused[l] != 0, H.maps[l], st, l, sym,
-                        fuse)) != cudaSuccess)
+                        fuse, false, &fresh)) != cudaSuccess)
             return e;
     }
     prof_end(s, coarse, st);
@@ -1737,7 +1808,9 @@ static cudaError_t enqueue_head64(Solver *s, cudaStream_t st)
 {
     const BoxSet<double> &S = s->h64.smooth[0];
     int sl = prof_begin(s, MG_PROF_PASS, st);
-    cudaError_t e = exch(s, S, 0, st);
+    // (the post-smoothing passes, and before the first cycle the prologue,
+    // leave the guard cells up to date; persistent launches do not)
+    cudaError_t e = level_persistent(s, s->h64, 0) ? exch(s, S, 0, st) : cudaSuccess;
     if (e != cudaSuccess) return e;
     e = launch_rbgs_pass_oop(S, s->active, 0, 0, s->partials, st);
     if (e != cudaSuccess) return e;
@@ -2204,6 +2277,7 @@ int solver_solve(Solver *s, const double *f, double *phi, double tol, mg_stats *
     CK(combine(s, s->dnormf, stream));
     if (!mixed && zero_guess) {
         // phi0 = 0: the starting residual is f itself
+        CK(exch(s, H.fine, 0, stream));   // (guard cells of an earlier solve)
         CK(cudaMemcpyAsync(s->dnorm, s->dnormf, sizeof(double) * nbox, cudaMemcpyDeviceToDevice,
                            stream));
     } else if (!mixed) {

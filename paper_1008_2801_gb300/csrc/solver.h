@@ -160,6 +160,9 @@ struct Solver {
     std::vector<const ExchRec *> xrec;               // [level] device exchange records
     std::vector<int> nxrec;                          // [level]
     std::vector<int> xmax;                           // [level] cells of the largest record
+    std::vector<std::vector<ExchRec>> recs;          // [level] the records on the host
+    char *pushmem = nullptr;                         // device: push tables (Box::prec)
+    std::vector<size_t> push64, push32;              // [level * nbox + box] offsets of the tables
     UnionBottom ub{};                                // union of the coarsest levels
 
     // set-up launch sets
