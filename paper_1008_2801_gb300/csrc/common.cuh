@@ -204,6 +204,7 @@ struct DescSet {
     int ntiles[TK_NKIND];
     int nbox;
     int flat;      // bit k: some box of the set tiles kind k flat (tile_flat)
+    int fold;      // some box's restriction applies the coarse level's first red pass (cinvD)
 };
 template <class T>
 using BoxSet = DescSet<Box<T>>;

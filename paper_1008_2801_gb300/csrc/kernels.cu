@@ -40,7 +40,7 @@ static inline cudaError_t counted(cudaError_t e)
 // environment launches them plainly.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-static bool pdl_enabled()
+bool pdl_enabled()
 {
     static const bool on = [] {
         const char *v = getenv("MG_PDL");
@@ -553,18 +553,20 @@ k_rbgs_sweep(BoxSet<T> S, const int *__restrict__ active, int src_is_phi2)
 // 0 already applied: -r / D on its red cells (the value of the pass's FMA
 // chain, whose products are all zero), which saves that pass: one of eight a
 // cycle on every coarse level, 17 us on 128^3, 3 to 4 on the small ones.
-template <class T>
+// FOLD: some box of the set folds (else the test costs the register-bound FP32
+// restriction a tenth).
+template <class T, bool FOLD>
 __device__ __forceinline__ void put_coarse(const Box<T> &B, int I, int J, int K, T r)
 {
     const long long cf = cfidx(B, I, J, K);
     B.fc[cf] = r;
     B.phic[(long long)K * B.cQ + (long long)J * B.cP + I] =
-        B.cinvD && !((I + J + K + B.cpar) & 1) ? -r * B.cinvD[cf] : T(0);
+        FOLD && B.cinvD && !((I + J + K + B.cpar) & 1) ? -r * B.cinvD[cf] : T(0);
 }
 
 // One coarse cell per thread, one tile of TK_COARSE: fc = mean over the 8
 // children of f - A phi, phic its start.
-template <class T, bool FC>
+template <class T, bool FC, bool FOLD>
 __device__ __forceinline__ void restrict_tile(const BoxSet<T> &S, const int *__restrict__ active,
                                               int t)
 {
@@ -594,19 +596,19 @@ __device__ __forceinline__ void restrict_tile(const BoxSet<T> &S, const int *__r
         return sum;
     };
     const T sum = B.D ? children(std::true_type{}) : children(std::false_type{});
-    put_coarse(B, I, J, K, sum * T(0.125));
+    put_coarse<T, FOLD>(B, I, J, K, sum * T(0.125));
 }
 
-template <class T, bool FC>
+template <class T, bool FC, bool FOLD>
 __global__ void __launch_bounds__(kThreads) k_resid_restrict(BoxSet<T> S, const int *__restrict__ active)
 {
     pdl_wait();
-    restrict_tile<T, FC>(S, active, blockIdx.x);
+    restrict_tile<T, FC, FOLD>(S, active, blockIdx.x);
 }
 
 // The red-children restriction of coarse cell (I, J, K); returns the sum of
 // the squared red residuals when NORM.
-template <class T, bool NORM>
+template <class T, bool NORM, bool FOLD>
 __device__ __forceinline__ T restrict_red_cell(const Box<T> &B, int I, int J, int K)
 {
     const int P = B.P;
@@ -636,7 +638,7 @@ __device__ __forceinline__ T restrict_red_cell(const Box<T> &B, int I, int J, in
                                : red4(std::true_type{}, std::false_type{}))
                       : (B.par ? red4(std::false_type{}, std::true_type{})
                                : red4(std::false_type{}, std::false_type{}));
-    put_coarse(B, I, J, K, sum * T(0.125));
+    put_coarse<T, FOLD>(B, I, J, K, sum * T(0.125));
     return r2;
 }
 
@@ -649,7 +651,7 @@ __device__ __forceinline__ T restrict_red_cell(const Box<T> &B, int I, int J, in
 // NORM: also each warp's sum of the squared red residuals into
 // partials[t * kThreads / 32 + warp] (hence ||f - A phi||^2 of the smoothed
 // iterate, summed per box in fixed order by the caller); no block barrier.
-template <class T, bool FC, bool NORM = false>
+template <class T, bool FC, bool NORM, bool FOLD>
 __device__ __forceinline__ void restrict_red_tile(const BoxSet<T> &S,
                                                   const int *__restrict__ active, int t,
                                                   double *__restrict__ partials = nullptr)
@@ -666,23 +668,23 @@ __device__ __forceinline__ void restrict_red_tile(const BoxSet<T> &S,
         // the warp's sum in T (for FP32 no FP64 adds on the narrow pipe; an
         // exit test's sum needs no more), widened once
         T r2 = T(0);
-        if (I < nx / 2 && J < ny / 2) r2 = restrict_red_cell<T, NORM>(B, I, J, K);
+        if (I < nx / 2 && J < ny / 2) r2 = restrict_red_cell<T, NORM, FOLD>(B, I, J, K);
         for (int o = 16; o > 0; o >>= 1) r2 += __shfl_down_sync(0xffffffffu, r2, o);
         const int tid = threadIdx.y * kTX + threadIdx.x;
         if ((tid & 31) == 0) partials[(long long)t * (kThreads / 32) + (tid >> 5)] = (double)r2;
         return;
     }
     if (I >= nx / 2 || J >= ny / 2) return;
-    restrict_red_cell<T, NORM>(B, I, J, K);
+    restrict_red_cell<T, NORM, FOLD>(B, I, J, K);
 }
 
-template <class T, bool FC, bool NORM>
+template <class T, bool FC, bool NORM, bool FOLD>
 __global__ void __launch_bounds__(kThreads) k_resid_restrict_red(BoxSet<T> S,
                                                                  const int *__restrict__ active,
                                                                  double *__restrict__ partials)
 {
     pdl_wait();
-    restrict_red_tile<T, FC, NORM>(S, active, blockIdx.x, partials);
+    restrict_red_tile<T, FC, NORM, FOLD>(S, active, blockIdx.x, partials);
 }
 
 // --------------------------------------------------------- prolongation ----
@@ -2975,14 +2977,14 @@ __global__ void __launch_bounds__(kThreads, 3) k_level_down(BoxSet<T> S, const i
     if (!exchange(0)) return;
     const int nc = S.ntiles[TK_COARSE];
     if (op.red && op.partials) {
-        if (op.flat) each(nc, [&](int t) { restrict_red_tile<T, true, true>(S, active, t, op.partials); });
-        else each(nc, [&](int t) { restrict_red_tile<T, false, true>(S, active, t, op.partials); });
+        if (op.flat) each(nc, [&](int t) { restrict_red_tile<T, true, true, true>(S, active, t, op.partials); });
+        else each(nc, [&](int t) { restrict_red_tile<T, false, true, true>(S, active, t, op.partials); });
     } else if (op.red) {
-        if (op.flat) each(nc, [&](int t) { restrict_red_tile<T, true>(S, active, t); });
-        else each(nc, [&](int t) { restrict_red_tile<T, false>(S, active, t); });
+        if (op.flat) each(nc, [&](int t) { restrict_red_tile<T, true, false, true>(S, active, t); });
+        else each(nc, [&](int t) { restrict_red_tile<T, false, false, true>(S, active, t); });
     } else {
-        if (op.flat) each(nc, [&](int t) { restrict_tile<T, true>(S, active, t); });
-        else each(nc, [&](int t) { restrict_tile<T, false>(S, active, t); });
+        if (op.flat) each(nc, [&](int t) { restrict_tile<T, true, true>(S, active, t); });
+        else each(nc, [&](int t) { restrict_tile<T, false, true>(S, active, t); });
     }
 }
 
@@ -3193,11 +3195,10 @@ template <class T>
 cudaError_t launch_resid_restrict(const BoxSet<T> &S, const int *active, cudaStream_t st)
 {
     if (S.ntiles[TK_COARSE] == 0) return cudaSuccess;
-    if (S.flat & (1 << TK_COARSE))
-        return pdl_launch(k_resid_restrict<T, true>, dim3(S.ntiles[TK_COARSE]), block2d(), 0, st,
-                          S, active);
-    return pdl_launch(k_resid_restrict<T, false>, dim3(S.ntiles[TK_COARSE]), block2d(), 0, st, S,
-                      active);
+    const bool flat = S.flat & (1 << TK_COARSE);
+    auto k = flat ? (S.fold ? k_resid_restrict<T, true, true> : k_resid_restrict<T, true, false>)
+                  : (S.fold ? k_resid_restrict<T, false, true> : k_resid_restrict<T, false, false>);
+    return pdl_launch(k, dim3(S.ntiles[TK_COARSE]), block2d(), 0, st, S, active);
 }
 
 template <class T>
@@ -3205,17 +3206,16 @@ cudaError_t launch_resid_restrict_red(const BoxSet<T> &S, const int *active, cud
                                       double *partials)
 {
     if (S.ntiles[TK_COARSE] == 0) return cudaSuccess;
-    const dim3 g(S.ntiles[TK_COARSE]);
     const bool flat = S.flat & (1 << TK_COARSE);
-    if (partials)
-        return flat ? pdl_launch(k_resid_restrict_red<T, true, true>, g, block2d(), 0, st, S,
-                                 active, partials)
-                    : pdl_launch(k_resid_restrict_red<T, false, true>, g, block2d(), 0, st, S,
-                                 active, partials);
-    return flat ? pdl_launch(k_resid_restrict_red<T, true, false>, g, block2d(), 0, st, S, active,
-                             partials)
-                : pdl_launch(k_resid_restrict_red<T, false, false>, g, block2d(), 0, st, S, active,
-                             partials);
+    auto pick = [&](auto norm, auto fold) {
+        constexpr bool N = decltype(norm)::value, F = decltype(fold)::value;
+        return flat ? k_resid_restrict_red<T, true, N, F> : k_resid_restrict_red<T, false, N, F>;
+    };
+    const std::true_type yes;
+    const std::false_type no;
+    auto k = partials ? (S.fold ? pick(yes, yes) : pick(yes, no))
+                      : (S.fold ? pick(no, yes) : pick(no, no));
+    return pdl_launch(k, dim3(S.ntiles[TK_COARSE]), block2d(), 0, st, S, active, partials);
 }
 
 cudaError_t launch_inner_judge(const BoxSet<float> &S, int *active32, const double *partials,

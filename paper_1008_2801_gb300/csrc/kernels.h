@@ -7,6 +7,8 @@ namespace mg {
 
 // Kernels launched by this library so far (all threads, all contexts).
 long long launch_counter();
+// Programmatic dependent launches are on (see kernels.cu).
+bool pdl_enabled();
 
 // ---- V-cycle stages over a set of boxes (one CTA per tile) --------------
 // `active` (nullable, indexed by Box::box) skips boxes whose flag is 0.

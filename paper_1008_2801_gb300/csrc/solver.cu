@@ -359,10 +359,14 @@ static void patch_set(const SetPlan<D> &p, char *dev)
 // CTAs run in waves of `slots` resident ones, so the sweep takes about
 // waves * (zc + 2) steps.  For each chunk count m the shortest chunk length
 // is ceil(nz / m) (equal chunks; a longer one only lengthens the critical
-// path); the m with the fewest steps wins.  Returns zc and its efficiency
-// (steps of useful plane work per resident slot over steps taken, 1 = perfect).
+// path); the m with the fewest steps wins.  The TMA-fed form's CTAs walk
+// several tiles each, and a tile costs it two steps more (its first two planes,
+// the change of tile): tma counts zc + 4, which takes 512^3 from 38 to 128
+// planes (591 -> 569 us a sweep) and leaves 256^3 at 37 (81 us; 64: 90).
+// Returns zc and the efficiency of the best zc + 2 count (steps of useful plane
+// work per resident slot over steps taken, 1 = perfect).
 template <class T>
-static int choose_zc(const std::vector<Box<T>> &boxes, long long slots, double *score)
+static int choose_zc(const std::vector<Box<T>> &boxes, long long slots, bool tma, double *score)
 {
     int maxnz = 1;
     double planes = 0.0;  // tile-planes of useful work
@@ -371,7 +375,7 @@ static int choose_zc(const std::vector<Box<T>> &boxes, long long slots, double *
         planes += (double)tiles_of(TK_SWEEP, B.nx, B.ny, B.nz, B.nz) * B.nz;
     }
     int best = std::min(kSweepZ, maxnz);
-    double best_cost = -1.0;
+    double best_cost = -1.0, plain_cost = -1.0;
     int last = -1;
     for (int m = 1; m <= maxnz; ++m) {
         const int Z = (maxnz + m - 1) / m;
@@ -380,13 +384,14 @@ static int choose_zc(const std::vector<Box<T>> &boxes, long long slots, double *
         long long ctas = 0;
         for (const auto &B : boxes) ctas += tiles_of(TK_SWEEP, B.nx, B.ny, B.nz, Z);
         const long long waves = (ctas + slots - 1) / slots;
-        const double cost = (double)waves * (Z + 2);
+        const double plain = (double)waves * (Z + 2), cost = (double)waves * (Z + (tma ? 4 : 2));
+        if (plain_cost < 0.0 || plain < plain_cost) plain_cost = plain;
         if (best_cost < 0.0 || cost < best_cost - 1e-9) {
             best_cost = cost;
             best = Z;
         }
     }
-    *score = planes / ((double)slots * best_cost);
+    *score = planes / ((double)slots * plain_cost);
     return best;
 }
 
@@ -570,7 +575,7 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
             if (l < H.lc[b]) set.push_back(make_box(s, H, b, l));
         if (!set.empty()) {
             double score = 0.0;
-            int zc = choose_zc(set, slots, &score);
+            int zc = choose_zc(set, slots, tma, &score);
             if (s->opts.sweep_zc > 0) {   // the tile depth given (autotuned) instead
                 int maxnz = 1;
                 for (const auto &B : set) maxnz = std::max(maxnz, B.nz);
@@ -611,6 +616,7 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
             }
         set_col_depth(s, set);
         plans.push_back(plan_set(blob, &H.smooth[l], set));
+        H.smooth[l].fold = l + 1 < (int)H.smooth.size() && H.red_done[l + 1];
     }
     H.njobs = (int)jobs.size();
     H.tail_zero = *std::min_element(H.lc.begin(), H.lc.end()) > 0;

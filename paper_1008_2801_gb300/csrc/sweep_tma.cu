@@ -12,20 +12,25 @@
 //     each stage guarded by a "full" mbarrier (the bytes landed) and an
 //     "empty" one (every consumer warp has read it);
 //   - warps 1..11, the consumers (8 row warps, 2 ring-row warps, 1
-//     ring-column warp): they wait only on the full barriers, meet at one
-//     named barrier per plane (between the red and the black updates), and
-//     release a plane's stage when they have read it.
-// Every operand address is a per-thread offset fixed at start plus a
-// compile-time stage and region constant: the plane loop is unrolled by the
-// number of stages, so a step's stage slots, ring slot and colour parity are
-// constants and the consumers issue few instructions per cell.  A step holds
-// three stages (planes k-1, k, k+1), so the other three are copies in
-// flight: 106 KB of shared memory and 71 registers give 2 CTAs (24 warps)
-// and six planes in flight per SM.  Measured at 512^3 (one launch, CUDA
-// events): 636 us per sweep, 75% of HBM, against 677 us with 4 stages and 3
-// CTAs per SM (one plane in flight per CTA), 980 us with 8 or 12 stages and
-// one CTA per SM (too few warps to hide the update chain) and 798 us for
-// the plain-load sweep.
+//     ring-column warp): they wait only on the full barriers, release a
+//     plane's stage when its operands are in registers, and meet at one named
+//     barrier per plane.
+// A consumer's lane owns a pair of cells of a column.  Whatever of the column
+// a step needs again stays in registers: the black values of planes k-1, k and
+// k+1 (one load a plane serves the red update above it, beside it and below
+// it), the z faces' weights, the black cell's f and weights (loaded with the red
+// cell's as one vector), and the column's own red values.  That took the shared
+// loads a row and plane from 27, all at a stride of two elements, to 13, half of
+// them vectors (L1 wavefronts 59% -> 38% of peak at 256^3), and a step's black
+// updates need no barrier after its red ones.  A step holds planes k and k+1,
+// so four stages are copies in flight; 100 KB of shared memory and 72 registers
+// give 2 CTAs (24 warps) per SM.  The CTAs are persistent: each walks tiles t,
+// t + grid, .. of the launch order, and the producer runs on into the next tile,
+// so a tile costs no pipeline ramp (a form whose CTAs took contiguous runs of
+// tiles lost the L2 reuse of tile halos).  Per sweep, 512^3: 637 -> 555 us (86%
+// of HBM on 24 bytes a cell), with the prolongation 801 -> 622 us; 256^3 96 ->
+// 80 us.  With the step's code unrolled over the stages the same kernel took 30
+// step bodies and waited for instructions (256^3: 113 us).
 // Waits are bounded: a wait that gives up sets the error word and the
 // threads go on (no consumer may leave the loop while the others meet at
 // the named barrier); the producer stops issuing, and before it exits it
@@ -37,6 +42,7 @@
 // (negative) coordinates, which read zeros.
 #include <cuda.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "kernels.h"
@@ -72,14 +78,12 @@ constexpr int kEcBytes = kEcW * kEcRows * 4;
 constexpr int kStageBytesP = kEcOff + pad128(kEcBytes);
 constexpr int kRedSW = 2 * kTX + 2, kRedPlane = (kSweepTY + 2) * kRedSW;   // red ring, floats
 
-// NS stages in the ring; the plane loop is unrolled by NS, so that every
-// stage and red-ring slot is a compile-time constant.  The red ring needs at
-// least 4 slots (planes k, k-1 and k-2 are read while the next step writes
-// the fourth) and a slot count dividing the unroll.
-__host__ __device__ constexpr int red_slots(int ns) { return ns % 4 == 0 ? 4 : ns; }
+// Two red planes: a step writes plane k's and reads plane k-1's, and ends at a
+// barrier.
+constexpr int kRedPlanes = 2;
 constexpr int smem_bytes(int ns, bool prol = false)
 {
-    return ns * (prol ? kStageBytesP : kStageBytes) + pad128(red_slots(ns) * kRedPlane * 4) + 128;
+    return ns * (prol ? kStageBytesP : kStageBytes) + pad128(kRedPlanes * kRedPlane * 4) + 128;
 }
 
 // the configuration the library launches: 6 stages, 2 CTAs (24 warps) per SM
@@ -177,14 +181,24 @@ __device__ __forceinline__ float red_update(float sw, float se, float ss, float 
     return s * __frcp_rn(((wxa + wxb) + (wya + wyb)) + (wza + wzb));
 }
 
-// step(kb, J) for J = I .. U-1 while kb + J <= z1 (step 0 always runs).
-template <int I, int U, class F>
-__device__ __forceinline__ void unroll_steps(F &step, int kb, int z1)
-{
-    if constexpr (I < U) {
-        if (I == 0 || kb + I <= z1) step(kb, std::integral_constant<int, I>{});
-        unroll_steps<I + 1, U>(step, kb, z1);
+// The next stage a consumer takes and the phase its plane lands in.
+template <int NS>
+struct Ring {
+    int s = 0;
+    unsigned par = 0;
+    __device__ __forceinline__ void next()
+    {
+        if (++s == NS) {
+            s = 0;
+            par ^= 1u;
+        }
     }
+};
+
+// Element of the staged coarse tile (40 x 6 cells) under column (x, y).
+__device__ __forceinline__ int coarse_at(int x, int y, int x0, int y0)
+{
+    return kEcOff / 4 + ((y >> 1) - (y0 >> 1) + 1) * kEcW + (x >> 1) - (x0 >> 1) + 4;
 }
 
 // PROL: the level's prolongation phi += e(parent) (the coarse correction,
@@ -202,9 +216,9 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
                      long long polls)
 {
     constexpr int STG = (PROL ? kStageBytesP : kStageBytes) / 4;   // stage stride, floats
-    constexpr int NR = red_slots(NS);
+    static_assert(NS >= 3, "planes k and k + 1 are held, another is in flight");
     constexpr int PHI = kSrcOff / 4, FF = kFOff / 4, WX = kWxOff / 4, WY = kWyOff / 4,
-                  WZ = kWzOff / 4, EC = kEcOff / 4, TW = kTileW, SW = kRedSW;
+                  WZ = kWzOff / 4, TW = kTileW, SW = kRedSW;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
@@ -212,28 +226,30 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
     float *const red = sm + NS * STG;
     __shared__ __align__(8) unsigned long long full[NS], empty[NS];
 
-    const int t = blockIdx.x;
     const int *ts = S.tstart[TK_SWEEP];
-    const int b = find_box(ts, S.nbox, t);
-    const Box<float> &B = S.boxes[b];
-    if (active && !active[B.box]) return;  // uniform over the CTA
-    const int nx = B.nx, ny = B.ny, nz = B.nz, P = B.P;
-    const long long Q = B.Q;
-    float *__restrict__ dst = src_is_phi2 ? B.phi : B.phi2;
-    const SweepMaps &M = maps[b];
-    const int zc = B.zc;
-    // the tile of the plain sweep's index space (2D tiles of 32 pairs x 8 rows)
-    int ex, ey, ez;
-    tile_extent(TK_SWEEP, nx, ny, nz, ex, ey, ez, zc);
-    const int ntx = (ex + kTX - 1) / kTX, nty = (ey + kSweepTY - 1) / kSweepTY;
-    int loc = t - ts[b];
-    const int tx = loc % ntx;
-    loc /= ntx;
-    const int ty = loc % nty;
-    const int tz = loc / nty;
-    const int x0 = tx * 2 * kTX, y0 = ty * kSweepTY;
-    const int z0 = tz * zc, z1 = min(z0 + zc, nz);
-    const int pfirst = z0 - 2, plast = z1 + 1;   // planes this CTA reads
+    const int ntile = S.ntiles[TK_SWEEP];
+    // tile t of the plain sweep's index space (2D tiles of 32 pairs x 8 rows);
+    // the box it belongs to is skipped when it is not active
+    struct Tile {
+        int b, x0, y0, z0, z1;
+        bool on;
+    };
+    auto tile_at = [&](int t) {
+        Tile T;
+        T.b = find_box(ts, S.nbox, t);
+        const Box<float> &B = S.boxes[T.b];
+        int ex, ey, ez;
+        tile_extent(TK_SWEEP, B.nx, B.ny, B.nz, ex, ey, ez, B.zc);
+        const int ntx = (ex + kTX - 1) / kTX, nty = (ey + kSweepTY - 1) / kSweepTY;
+        int loc = t - ts[T.b];
+        T.x0 = loc % ntx * 2 * kTX;
+        loc /= ntx;
+        T.y0 = loc % nty * kSweepTY;
+        T.z0 = loc / nty * B.zc;
+        T.z1 = min(T.z0 + B.zc, B.nz);
+        T.on = !active || active[B.box];
+        return T;
+    };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < NS; ++s) {
@@ -243,185 +259,300 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 
     if (warp == 0) {
-        // producer: plane p goes to stage (p - pfirst) % NS; from plane
-        // pfirst + NS on it waits until the consumers have released the stage
+        // producer: the i-th plane of this CTA's tiles goes to stage i % NS;
+        // from the NS-th on it waits until the consumers have released the
+        // stage.  It runs on into the next tile while they finish this one.
         if (lane == 0) {
-            for (int i = 0; i < (PROL ? 7 : 6); ++i) tensormap_acquire(&M.m[i]);
-            const CUtensorMap *msrc = &M.m[src_is_phi2 ? 1 : 0];
-            int last = pfirst - 1;
-            for (int p = pfirst; p <= plast; ++p) {
-                const int i = p - pfirst, s = i % NS;
-                if (i >= NS &&
-                    !mbar_wait(smem_addr(&empty[s]), (unsigned)(((i / NS) - 1) & 1), polls)) {
-                    atomicExch(err, 1);
-                    break;
+            int i = 0, mapped = -1;
+            bool ok = true;
+            for (int t = blockIdx.x; ok && t < ntile; t += gridDim.x) {
+                const Tile T = tile_at(t);
+                if (!T.on) continue;
+                const SweepMaps &M = maps[T.b];
+                if (T.b != mapped) {
+                    for (int m = 0; m < (PROL ? 7 : 6); ++m) tensormap_acquire(&M.m[m]);
+                    mapped = T.b;
                 }
-                last = p;
-                unsigned char *base = smem + s * (STG * 4);
-                const unsigned bar = smem_addr(&full[s]);
-                mbar_expect_tx(bar, kTxBytes + (PROL ? kEcBytes : 0));
-                const int zt = p + 1;  // tensor z of logical plane p (guard plane first)
-                tma_load_3d(smem_addr(base + kSrcOff), msrc, bar, x0 - 4, y0 - 2, zt);
-                tma_load_3d(smem_addr(base + kFOff), &M.m[2], bar, x0 - 4, y0 - 1, zt);
-                tma_load_3d(smem_addr(base + kWxOff), &M.m[3], bar, x0 - 4, y0 - 1, zt);
-                tma_load_3d(smem_addr(base + kWyOff), &M.m[4], bar, x0 - 4, y0 - 1, zt);
-                tma_load_3d(smem_addr(base + kWzOff), &M.m[5], bar, x0 - 4, y0 - 1, zt);
-                // the coarse correction under plane p: coarse plane p >> 1
-                // (planes -1, -2: the coarse guard plane, zero)
-                if (PROL)
-                    tma_load_3d(smem_addr(base + kEcOff), &M.m[6], bar, x0 / 2 - 4, y0 / 2 - 1,
-                                (p >> 1) + 1);
+                const CUtensorMap *msrc = &M.m[src_is_phi2 ? 1 : 0];
+                const int x0 = T.x0, y0 = T.y0;
+                for (int p = T.z0 - 2; p <= T.z1 + 1; ++p, ++i) {
+                    const int s = i % NS;
+                    if (i >= NS &&
+                        !mbar_wait(smem_addr(&empty[s]), (unsigned)(((i / NS) - 1) & 1), polls)) {
+                        atomicExch(err, 1);
+                        ok = false;
+                        break;
+                    }
+                    unsigned char *base = smem + s * (STG * 4);
+                    const unsigned bar = smem_addr(&full[s]);
+                    mbar_expect_tx(bar, kTxBytes + (PROL ? kEcBytes : 0));
+                    const int zt = p + 1;  // tensor z of logical plane p (guard plane first)
+                    tma_load_3d(smem_addr(base + kSrcOff), msrc, bar, x0 - 4, y0 - 2, zt);
+                    tma_load_3d(smem_addr(base + kFOff), &M.m[2], bar, x0 - 4, y0 - 1, zt);
+                    tma_load_3d(smem_addr(base + kWxOff), &M.m[3], bar, x0 - 4, y0 - 1, zt);
+                    tma_load_3d(smem_addr(base + kWyOff), &M.m[4], bar, x0 - 4, y0 - 1, zt);
+                    tma_load_3d(smem_addr(base + kWzOff), &M.m[5], bar, x0 - 4, y0 - 1, zt);
+                    // the coarse correction under plane p: coarse plane p >> 1
+                    // (planes -1, -2: the coarse guard plane, zero)
+                    if (PROL)
+                        tma_load_3d(smem_addr(base + kEcOff), &M.m[6], bar, x0 / 2 - 4,
+                                    y0 / 2 - 1, (p >> 1) + 1);
+                }
             }
             // every copy issued has landed before this thread exits (the
             // earlier planes' stages were waited on before their reuse)
-            for (int p = max(pfirst, last - NS + 1); p <= last; ++p)
-                if (!mbar_wait(smem_addr(&full[(p - pfirst) % NS]),
-                               (unsigned)(((p - pfirst) / NS) & 1), kWaitLimit))
+            for (int q = max(0, i - NS); q < i; ++q)
+                if (!mbar_wait(smem_addr(&full[q % NS]), (unsigned)((q / NS) & 1), kWaitLimit))
                     atomicExch(err, 1);
         }
         return;
     }
 
-
     // consumers
     const int cw = warp - 1;           // 0..7 row warps, 8 / 9 ring rows, 10 ring column
-    const bool own = cw < kSweepTY;
-    const bool colw = cw == kSweepTY + 2;
-    const int xa = x0 + 2 * lane;
-    // this thread's red cell for the two colour parities q: x or y, the
-    // staged-operand offsets (phi region, operand regions), the ring slot
-    // position and validity
-    int qy = 0;            // row warps: y + k decides q; ring column: x + y0 + k
-    int phiC[2], opC[2], ringC[2];
-    bool valid[2];
-    bool ractive;
-    // PROL: offsets in the coarse tile of the parents of the red cell's
-    // west, east, south and north neighbours and of its own column (the
-    // parent of its z neighbours, in their planes' tiles)
-    int eW[2], eE[2], eS[2], eN[2], eC[2];
-    auto ecoarse = [&](int x, int y) {
-        return ((y >> 1) - (y0 >> 1) + 1) * kEcW + (x >> 1) - (x0 >> 1) + 4;
+    Ring<NS> rg;
+    long long left = polls;
+    auto take = [&]() {   // the next plane's stage, once the plane has landed in it
+        const int st = rg.s;
+        if (!mbar_wait(smem_addr(&full[st]), rg.par, left)) {
+            if (lane == 0) atomicExch(err, 1);
+            left = 0;     // (a wait that gave up is not repeated)
+        }
+        rg.next();
+        return st;
     };
-    auto parents = [&](int q, int x, int y) {
-        eW[q] = ecoarse(x - 1, y);
-        eE[q] = ecoarse(x + 1, y);
-        eS[q] = ecoarse(x, y - 1);
-        eN[q] = ecoarse(x, y + 1);
-        eC[q] = ecoarse(x, y);
-    };
-    if (!colw) {
-        const int y = own ? y0 + cw : cw == kSweepTY ? y0 - 1 : y0 + kSweepTY;
-        const int srow = own ? cw + 1 : cw == kSweepTY ? 0 : kSweepTY + 1;
-        qy = y;
-        for (int q = 0; q < 2; ++q) {
-            const int x = xa + q;
-            phiC[q] = (y - y0 + 2) * TW + (x - x0 + 4);
-            opC[q] = (y - y0 + 1) * TW + (x - x0 + 4);
-            ringC[q] = srow * SW + x - x0 + 1;
-            valid[q] = y >= 0 && y < ny && x < nx;
-            parents(q, x, y);
-        }
-        ractive = true;
-    } else {
-        const int xc = lane < kSweepTY / 2 ? x0 - 1 : x0 + 2 * kTX;
-        qy = xc + y0;
-        for (int q = 0; q < 2; ++q) {
-            const int yy = y0 + 2 * (lane % (kSweepTY / 2)) + q;
-            phiC[q] = (yy - y0 + 2) * TW + (xc - x0 + 4);
-            opC[q] = (yy - y0 + 1) * TW + (xc - x0 + 4);
-            ringC[q] = (yy - y0 + 1) * SW + xc - x0 + 1;
-            valid[q] = lane < kSweepTY && xc >= 0 && xc < nx && yy < ny;
-            parents(q, xc, yy);
-        }
-        ractive = lane < kSweepTY;
-    }
-    // row warps: the pair (xa, xa + 1) of row yo
-    const int yo = y0 + cw;
-    const bool orow = own && yo < ny;
-    const int pairC = (cw + 1) * SW + 2 * lane + 1;   // ring position of xa
-    const int bopC = (cw + 1) * TW + 2 * lane + 4;    // operand position of xa
-    const bool fullp = xa + 1 < nx, halfp = xa < nx;
-    float *gdst = dst + (long long)(z0 - 2) * Q + (long long)yo * P + xa;   // plane kb - 1
-
-    auto step = [&](int kb, auto J) {
-        constexpr int j = decltype(J)::value;
-        // plane k = kb + j: stages of planes k-1, k, k+1, ring slots of k, k-1, k-2
-        constexpr int sM = j % NS, s0 = (j + 1) % NS, sP = (j + 2) % NS;
-        constexpr int r0 = j % NR, rm = (j + NR - 1) % NR, rmm = (j + NR - 2) % NR;
-        const int k = kb + j;
-        if (!mbar_wait(smem_addr(&full[sP]), (unsigned)(((k + 1 - pfirst) / NS) & 1),
-                       polls) &&
-            lane == 0)
-            atomicExch(err, 1);
-        const float *SM_ = sm + sM * STG, *S0 = sm + s0 * STG, *SP = sm + sP * STG;
-        float *R0 = red + r0 * kRedPlane;
-        // (1) red values of plane k: own columns, and the ring inside the chunk
-        if (ractive && (own || (k >= z0 && k < z1))) {
-            const int q = (qy + k) & 1;
-            const int c = q ? phiC[1] : phiC[0];
-            const int o = q ? opC[1] : opC[0];
-            const bool v = (q ? valid[1] : valid[0]) && k >= 0 && k < nz;
-            float nw = S0[PHI + c - 1], ne = S0[PHI + c + 1], ns = S0[PHI + c - TW],
-                  nn = S0[PHI + c + TW], nd = SM_[PHI + c], nu = SP[PHI + c];
-            if (PROL) {   // the neighbours as the prolongation leaves them
-                nw += S0[EC + (q ? eW[1] : eW[0])];
-                ne += S0[EC + (q ? eE[1] : eE[0])];
-                ns += S0[EC + (q ? eS[1] : eS[0])];
-                nn += S0[EC + (q ? eN[1] : eN[0])];
-                nd += SM_[EC + (q ? eC[1] : eC[0])];
-                nu += SP[EC + (q ? eC[1] : eC[0])];
-            }
-            const float val = red_update(nw, ne, ns, nn, nd, nu, S0[WX + o], S0[WX + o + 1],
-                                         S0[WY + o], S0[WY + o + TW], S0[WZ + o], SP[WZ + o],
-                                         S0[FF + o]);
-            R0[q ? ringC[1] : ringC[0]] = v ? val : 0.f;
-        }
-        named_barrier(1, 32 * kConsumers);
-        // (2) black values of plane k-1 and the pair store (row warps)
-        const int km = k - 1;
-        if (orow && km >= z0 && km < z1) {
-            const float *Rm = red + rm * kRedPlane, *Rmm = red + rmm * kRedPlane;
-            const int pm = (yo + km) & 1;   // red parity at plane k-1
-            const int xb = xa + (pm ^ 1);
-            const int lb = pairC + (pm ^ 1), ob = bopC + (pm ^ 1);
-            const float rv = Rm[pairC + pm];
-            float bv = 0.f;
-            if (xb < nx) {
-                const float wxa = SM_[WX + ob], wxb = SM_[WX + ob + 1];
-                const float wya = SM_[WY + ob], wyb = SM_[WY + ob + TW];
-                const float wza = SM_[WZ + ob], wzb = S0[WZ + ob];
-                float s = fmaf(wxa, Rm[lb - 1], -SM_[FF + ob]);
-                s = fmaf(wxb, Rm[lb + 1], s);
-                s = fmaf(wya, Rm[lb - SW], s);
-                s = fmaf(wyb, Rm[lb + SW], s);
-                s = fmaf(wza, Rmm[lb], s);
-                s = fmaf(wzb, R0[lb], s);
-                bv = s * __frcp_rn(((wxa + wxb) + (wya + wyb)) + (wza + wzb));
-            }
-            const float va = pm ? bv : rv, vb = pm ? rv : bv;
-            float *g = gdst + (long long)j * Q;
-            if (fullp) {
-                float2 v2;
-                v2.x = va;
-                v2.y = vb;
-                *reinterpret_cast<float2 *>(g) = v2;
-            } else if (halfp) {
-                g[0] = va;
-            }
-        }
-        // (3) plane k-1 is read: release its stage
+    auto release = [&](int stage) {            // this warp has read the stage's plane
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_addr(&empty[sM]));
+        if (lane == 0) mbar_arrive(smem_addr(&empty[stage]));
     };
-    // the first step also needs planes pfirst and pfirst + 1
-    if (!(mbar_wait(smem_addr(&full[0]), 0u, polls) &&
-          mbar_wait(smem_addr(&full[1]), 0u, polls)) &&
-        lane == 0)
-        atomicExch(err, 1);
-    for (int kb = z0 - 1; kb <= z1; kb += NS, gdst += NS * Q)
-        unroll_steps<0, NS>(step, kb, z1);
+    int r0 = 0;   // where the current plane's red values go
+
+    if (cw < kSweepTY + 2) {
+        // Rows y0 - 1 .. y0 + 8: lane owns the pair (xa, xa + 1), whose red cell
+        // on plane k is at position q = (y + k) & 1.  A row's q is uniform and
+        // the planes alternate, so the loop holds a step for either q, with
+        // every position a constant (unrolled over the stages as well, the row
+        // kinds and parities made 30 step bodies, and the warps waited for
+        // instructions).
+        auto march = [&](auto own_tag) {
+            constexpr bool OWN = decltype(own_tag)::value;   // row of the tile: black cells too
+            const int row = OWN ? cw + 1 : cw == kSweepTY ? 0 : kSweepTY + 1;   // 0 .. 9
+            const int pa = (row + 1) * TW + 2 * lane + 4;    // phi region, of xa
+            const int oa = row * TW + 2 * lane + 4;          // operand regions
+            const int ra = row * SW + 2 * lane + 1;          // red plane
+            for (int t = blockIdx.x; t < ntile; t += gridDim.x) {
+            const Tile T = tile_at(t);
+            if (!T.on) continue;
+            const Box<float> &B = S.boxes[T.b];
+            const int nx = B.nx, ny = B.ny, nz = B.nz, z0 = T.z0, z1 = T.z1;
+            const long long Q = B.Q;
+            const int y = T.y0 + row - 1, xa = T.x0 + 2 * lane;
+            const bool vy = y >= 0 && y < ny;
+            const bool v0 = vy && xa < nx, v1 = vy && xa + 1 < nx;
+            const int ec = coarse_at(xa, y, T.x0, T.y0), es = coarse_at(xa, y - 1, T.x0, T.y0),
+                      en = coarse_at(xa, y + 1, T.x0, T.y0);
+            const bool orow = OWN && y < ny;
+            float *gdst = (src_is_phi2 ? B.phi : B.phi2) + (long long)(z0 - 2) * Q +
+                          (long long)y * B.P + xa;           // plane k - 1
+            const int q0 = (y + z0 - 1) & 1;
+            // planes z0 - 2 and z0 - 1; then a step takes plane k + 1
+            const int sA = take();
+            int s0 = take();
+            const float *const A = sm + sA * STG, *const A1 = sm + s0 * STG;
+            // carried over the steps, all of this column: the black values of
+            // planes k - 1 (under the red cell) and k (beside it), the z-face
+            // weights of plane k; of plane k - 1 the black cell's f and weights,
+            // and the red values of planes k - 1 and k - 2
+            float dn = A[PHI + pa + q0], be = A1[PHI + pa + 1 - q0];
+            if (PROL) {
+                dn += A[ec];
+                be += A1[ec];
+            }
+            float2 wz = *reinterpret_cast<const float2 *>(A1 + WZ + oa);
+            float fB = 0.f, xB0 = 0.f, xB1 = 0.f, yB0 = 0.f, yB1 = 0.f, zB0 = 0.f;
+            float r1 = 0.f, r2 = 0.f;
+            release(sA);
+            int k = z0 - 1;
+            auto step = [&](auto q_tag) {
+                constexpr int q = decltype(q_tag)::value;
+                const int sP = take();
+                const float *const S0 = sm + s0 * STG, *const SP = sm + sP * STG;
+                float *const R0 = red + r0;
+                const float *const R1 = red + (kRedPlane - r0);
+                // operands of plane k (the red cell's now, the black cell's on
+                // the next step) and the black value above
+                float up = SP[PHI + pa + q], outer = S0[PHI + pa + (q ? 2 : -1)],
+                      so = S0[PHI + pa + q - TW], no = S0[PHI + pa + q + TW];
+                if (PROL) {   // the neighbours as the prolongation leaves them
+                    up += SP[ec];
+                    outer += S0[ec + (q ? 1 : -1)];
+                    so += S0[es];
+                    no += S0[en];
+                }
+                float fR, x0w, x1w, y0w, y1w, z1w;   // the red cell's
+                float fN = 0.f, x0n = 0.f, x1n = 0.f, y0n = 0.f, y1n = 0.f;   // the black cell's
+                float2 wzn;
+                if constexpr (OWN) {
+                    const float2 f2 = *reinterpret_cast<const float2 *>(S0 + FF + oa);
+                    const float2 wx = *reinterpret_cast<const float2 *>(S0 + WX + oa);
+                    const float wx2 = S0[WX + oa + 2];
+                    const float2 wy = *reinterpret_cast<const float2 *>(S0 + WY + oa);
+                    const float2 wyu = *reinterpret_cast<const float2 *>(S0 + WY + oa + TW);
+                    wzn = *reinterpret_cast<const float2 *>(SP + WZ + oa);
+                    fR = q ? f2.y : f2.x;
+                    x0w = q ? wx.y : wx.x;
+                    x1w = q ? wx2 : wx.y;
+                    y0w = q ? wy.y : wy.x;
+                    y1w = q ? wyu.y : wyu.x;
+                    fN = q ? f2.x : f2.y;
+                    x0n = q ? wx.x : wx.y;
+                    x1n = q ? wx.y : wx2;
+                    y0n = q ? wy.x : wy.y;
+                    y1n = q ? wyu.x : wyu.y;
+                } else {
+                    fR = S0[FF + oa + q];
+                    x0w = S0[WX + oa + q];
+                    x1w = S0[WX + oa + q + 1];
+                    y0w = S0[WY + oa + q];
+                    y1w = S0[WY + oa + q + TW];
+                    wzn = *reinterpret_cast<const float2 *>(SP + WZ + oa);
+                }
+                z1w = q ? wzn.y : wzn.x;
+                const float z0w = q ? wz.y : wz.x;   // also the black cell's upper face
+                // the black neighbours of plane k - 1's black cell: red values
+                // published by the barrier of the last step
+                float ob = 0.f, sb = 0.f, nb = 0.f;
+                if constexpr (OWN) {
+                    ob = R1[ra + (q ? 2 : -1)];
+                    sb = R1[ra + q - SW];
+                    nb = R1[ra + q + SW];
+                }
+                release(s0);   // every operand is in registers
+                // (1) the red value of plane k
+                float val = red_update(q ? be : outer, q ? outer : be, so, no, dn, up, x0w, x1w,
+                                       y0w, y1w, z0w, z1w, fR);
+                val = (q ? v1 : v0) && k >= 0 && k < nz ? val : 0.f;
+                R0[ra + q] = val;
+                // (2) the black value of plane k - 1, at the same position: its
+                // neighbour in the pair and those above and below are this
+                // thread's own red values
+                if constexpr (OWN) {
+                    const int km = k - 1;
+                    if (orow && km >= z0 && km < z1) {
+                        float bv = red_update(q ? r1 : ob, q ? ob : r1, sb, nb, r2, val, xB0, xB1,
+                                              yB0, yB1, zB0, z0w, fB);
+                        bv = (q ? v1 : v0) ? bv : 0.f;
+                        if (v1) {
+                            float2 o;
+                            o.x = q ? r1 : bv;
+                            o.y = q ? bv : r1;
+                            *reinterpret_cast<float2 *>(gdst) = o;
+                        } else if (v0) {
+                            gdst[0] = q ? r1 : bv;
+                        }
+                    }
+                    fB = fN;
+                    xB0 = x0n;
+                    xB1 = x1n;
+                    yB0 = y0n;
+                    yB1 = y1n;
+                    zB0 = q ? wz.x : wz.y;   // plane k's lower face at its black cell
+                    r2 = r1;
+                    r1 = val;
+                }
+                dn = be;
+                be = up;
+                wz = wzn;
+                named_barrier(1, 32 * kConsumers);
+                s0 = sP;
+                r0 = kRedPlane - r0;
+                gdst += Q;
+                ++k;
+            };
+            bool second = q0 != 0;   // the first step's plane has q = 1
+            while (true) {
+                if (!second) {
+                    step(std::integral_constant<int, 0>{});
+                    if (k > z1) break;
+                }
+                second = false;
+                step(std::integral_constant<int, 1>{});
+                if (k > z1) break;
+            }
+            release(s0);   // plane z1 + 1
+            }
+        };
+        if (cw < kSweepTY) march(std::true_type{});
+        else march(std::false_type{});
+        return;
+    }
+
+    // the ring columns x0 - 1 (lanes 0..3) and x0 + 64 (lanes 4..7): a lane owns
+    // the pair (yy, yy + 1), red at position q = (xc + y0 + k) & 1
+    const bool on = lane < kSweepTY;
+    const int cx = lane < kSweepTY / 2 ? -1 : 2 * kTX, cy = 2 * (lane % (kSweepTY / 2));
+    const int pc = (cy + 2) * TW + cx + 4, oc = pc - TW, rc = (cy + 1) * SW + cx + 1;
+    for (int t = blockIdx.x; t < ntile; t += gridDim.x) {
+        const Tile T = tile_at(t);
+        if (!T.on) continue;
+        const Box<float> &B = S.boxes[T.b];
+        const int nz = B.nz, z0 = T.z0, z1 = T.z1;
+        const int xc = T.x0 + cx, yy = T.y0 + cy;
+        const bool vx = on && xc >= 0 && xc < B.nx;
+        const bool v0 = vx && yy < B.ny, v1 = vx && yy + 1 < B.ny;
+        // (the parents of a pair's rows are one row of the coarse tile)
+        const int ec = coarse_at(xc, yy, T.x0, T.y0), ew = coarse_at(xc - 1, yy, T.x0, T.y0),
+                  ee = coarse_at(xc + 1, yy, T.x0, T.y0);
+        int q = (xc + T.y0 + z0 - 1) & 1;
+        const int sA = take();
+        int s0 = take();
+        float dn = 0.f, be = 0.f;
+        if (on) {
+            const float *const A = sm + sA * STG, *const A1 = sm + s0 * STG;
+            dn = A[PHI + pc + q * TW];
+            be = A1[PHI + pc + (1 - q) * TW];
+            if (PROL) {
+                dn += A[ec];
+                be += A1[ec];
+            }
+        }
+        release(sA);
+        for (int k = z0 - 1; k <= z1; ++k) {
+            const int sP = take();
+            const float *const S0 = sm + s0 * STG, *const SP = sm + sP * STG;
+            float *const R0 = red + r0;
+            if (on) {
+                const int c = pc + q * TW, o = oc + q * TW;
+                float up = SP[PHI + c];
+                if (PROL) up += SP[ec];
+                if (k >= z0 && k < z1) {
+                    float we = S0[PHI + c - 1], ea = S0[PHI + c + 1],
+                          out = S0[PHI + pc + (q ? 2 * TW : -TW)];
+                    if (PROL) {
+                        we += S0[ew];
+                        ea += S0[ee];
+                        out += S0[ec + (q ? kEcW : -kEcW)];
+                    }
+                    const float val =
+                        red_update(we, ea, q ? be : out, q ? out : be, dn, up, S0[WX + o],
+                                   S0[WX + o + 1], S0[WY + o], S0[WY + o + TW], S0[WZ + o],
+                                   SP[WZ + o], S0[FF + o]);
+                    R0[rc + q * SW] = (q ? v1 : v0) && k >= 0 && k < nz ? val : 0.f;
+                }
+                dn = be;
+                be = up;
+            }
+            q ^= 1;
+            release(s0);
+            named_barrier(1, 32 * kConsumers);
+            s0 = sP;
+            r0 = kRedPlane - r0;
+        }
+        release(s0);   // plane z1 + 1
+    }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
@@ -536,6 +667,25 @@ int sweep_tma_ctas_per_sm()
     return n > 0 ? n : 1;
 }
 
+// CTAs that fit on the current device at once.
+static int resident_ctas()
+{
+    constexpr int kMaxDevices = 64;
+    static std::mutex mu;
+    static int known[kMaxDevices] = {};
+    int dev = 0, sms = 1;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+    std::lock_guard<std::mutex> lk(mu);
+    if (dev >= 0 && dev < kMaxDevices && known[dev]) return known[dev];
+    if (dev < 0 || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    const int n = sms * sweep_tma_ctas_per_sm();
+    if (dev < kMaxDevices) known[dev] = n;
+    return n;
+}
+
 long long sweep_wait_polls(int wait_limit)
 {
     return wait_limit == 0 ? kWaitLimit : wait_limit < 0 ? 0 : (long long)wait_limit;
@@ -546,18 +696,24 @@ cudaError_t launch_rbgs_sweep_tma(const BoxSet<float> &S, const SweepMaps *maps,
                                   bool prolong)
 {
     if (S.ntiles[TK_SWEEP] == 0) return cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(std::min(S.ntiles[TK_SWEEP], resident_ctas()));
+    cfg.blockDim = dim3(kTmaThreads);
+    cfg.dynamicSmemBytes = smem_bytes(kStages, prolong);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl_enabled() ? 1 : 0;
     if (prolong) {
         set_smem_attributes<kStages, kMinCtas, true>();
-        k_rbgs_sweep_tma<kStages, kMinCtas, true>
-            <<<S.ntiles[TK_SWEEP], kTmaThreads, smem_bytes(kStages, true), st>>>(
-                S, maps, active, src_is_phi2, err, wait_polls);
-    } else {
-        set_smem_attributes<kStages, kMinCtas, false>();
-        k_rbgs_sweep_tma<kStages, kMinCtas, false>
-            <<<S.ntiles[TK_SWEEP], kTmaThreads, smem_bytes(kStages), st>>>(
-                S, maps, active, src_is_phi2, err, wait_polls);
+        return cudaLaunchKernelEx(&cfg, k_rbgs_sweep_tma<kStages, kMinCtas, true>, S, maps, active,
+                                  src_is_phi2, err, wait_polls);
     }
-    return cudaGetLastError();
+    set_smem_attributes<kStages, kMinCtas, false>();
+    return cudaLaunchKernelEx(&cfg, k_rbgs_sweep_tma<kStages, kMinCtas, false>, S, maps, active,
+                              src_is_phi2, err, wait_polls);
 }
 
 }  // namespace mg
