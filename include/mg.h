@@ -137,10 +137,8 @@ typedef struct {
     int tma;          /* 0 (default) or 1: FP32 fused sweeps are fed by the
                          Tensor Memory Accelerator: a producer warp copies
                          each plane's tiles into a shared-memory ring that
-                         eleven consumer warps compute from (on levels
-                         whose rows and planes hold a whole 72 x 12 copy
-                         box, when the driver can encode tensor maps;
-                         elsewhere plain loads); -1: every fused sweep
+                         eleven consumer warps compute from (when the driver
+                         can encode tensor maps; else plain loads); -1: every fused sweep
                          reads its operands with plain loads.  Both give
                          bitwise the same result */
     int krylov;       /* 0 (default): the iteration is V-cycles (FP64) or
@@ -182,7 +180,7 @@ typedef struct {
                          per-stage launches.  Levels smoothed with fused
                          FP32 sweeps keep their own launches. */
     int sweep_zc;     /* tile depth of the fused FP32 sweep: planes of z a
-                         CTA marches through (its tile is 64 x 8 cells in
+                         CTA marches through (its tile is 64 x 8 or 32 x 16 cells in
                          x, y).  0 (default): chosen by a model that fills
                          whole waves of resident CTAs; n in 1..4096: n */
     int level_ctas;   /* persistent = 1: CTAs per SM of the persistent

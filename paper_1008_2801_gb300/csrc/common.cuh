@@ -90,6 +90,7 @@ struct Box {
     int box;         // index of the box in its batch
     int zc;          // planes per CTA of the fused sweep (chosen on the host)
     int cd;          // planes per thread of the column kernels (0: kColZ; see col_depth)
+    int sw;          // width of the fused sweep's tiles: 32, or 64 (0)
     int par;         // colour of local cell (0,0,0): (sum of the box's lower corner) % 2 on a
                      // coupled level (red = global i+j+k even), else 0
     int rb;          // 1: f, invD and D are colour-split (see split_at); 0: natural layout
@@ -182,8 +183,10 @@ inline __host__ __device__ bool tile_flat(int kind, int ex)
 }
 
 inline __host__ __device__ int tiles_of(int kind, int nx, int ny, int nz, int zc = kSweepZ,
-                                        int cd = kColZ)
+                                        int cd = kColZ, int sw = 64)
 {
+    if (kind == TK_SWEEP && sw == 32)   // the TMA sweep's 32 x 16 tiles
+        return ((nx + 31) / 32) * ((ny + 15) / 16) * ((nz + zc - 1) / zc);
     int ex, ey, ez;
     tile_extent(kind, nx, ny, nz, ex, ey, ez, zc, cd);
     const int ty = tile_rows(kind);
@@ -204,6 +207,7 @@ struct DescSet {
     int ntiles[TK_NKIND];
     int nbox;
     int flat;      // bit k: some box of the set tiles kind k flat (tile_flat)
+    int sweep_w;   // width of the TMA sweep's tiles: 32, or 64 (0)
     int fold;      // some box's restriction applies the coarse level's first red pass (cinvD)
 };
 template <class T>

@@ -46,7 +46,8 @@ bool sweep_tma_prol_fits(int nx, int ny, int cx, int cy);
 bool encode_sweep_maps(SweepMaps *out, int nx, int ny, int nz, const float *phi_base,
                        const float *phi2_base, const float *f_base, const float *wx_base,
                        const float *wy_base, const float *wz_base,
-                       const float *phic_base = nullptr, int cx = 0, int cy = 0, int cz = 0);
+                       const float *phic_base = nullptr, int cx = 0, int cy = 0, int cz = 0,
+                       int width = 64);
 int sweep_tma_ctas_per_sm();
 // Same result as launch_rbgs_sweep<float>; *err is set to 1 if a bounded
 // wait on a tile copy gave up after wait_polls polls (the CTA then waits,

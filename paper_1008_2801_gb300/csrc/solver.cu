@@ -322,6 +322,9 @@ static void set_col_depth(const Solver *s, std::vector<Box<T>> &boxes)
 template <class T>
 static int cd_of(const Box<T> &B) { return col_depth(B); }
 static int cd_of(const SetupBox &) { return kColZ; }
+template <class T>
+static int sw_of(const Box<T> &B) { return B.sw ? B.sw : 64; }
+static int sw_of(const SetupBox &) { return 64; }
 
 template <class D>
 static SetPlan<D> plan_set(DescBlob &blob, DescSet<D> *target, const std::vector<D> &boxes)
@@ -335,11 +338,13 @@ static SetPlan<D> plan_set(DescBlob &blob, DescSet<D> *target, const std::vector
         std::vector<int> ts(boxes.size() + 1, 0);
         for (size_t i = 0; i < boxes.size(); ++i) {
             const int zc = boxes[i].zc > 0 ? boxes[i].zc : kSweepZ;
-            ts[i + 1] = ts[i] + tiles_of(k, boxes[i].nx, boxes[i].ny, boxes[i].nz, zc, cd_of(boxes[i]));
+            ts[i + 1] = ts[i] + tiles_of(k, boxes[i].nx, boxes[i].ny, boxes[i].nz, zc, cd_of(boxes[i]),
+                                       sw_of(boxes[i]));
             int ex, ey, ez;
             tile_extent(k, boxes[i].nx, boxes[i].ny, boxes[i].nz, ex, ey, ez, zc);
             if (tile_flat(k, ex)) target->flat |= 1 << k;
         }
+        if (!boxes.empty() && sw_of(boxes[0]) == 32) target->sweep_w = 32;
         target->ntiles[k] = ts.back();
         p.ts_off[k] = blob.put(ts.data(), ts.size() * sizeof(int));
     }
@@ -363,16 +368,26 @@ static void patch_set(const SetPlan<D> &p, char *dev)
 // several tiles each, and a tile costs it two steps more (its first two planes,
 // the change of tile): tma counts zc + 4, which takes 512^3 from 38 to 128
 // planes (591 -> 569 us a sweep) and leaves 256^3 at 37 (81 us; 64: 90).
+// width: of the tiles; *steps: of the choice.
+// A box takes equal chunks of at most zc planes (box_zc), so that the boxes of a
+// batch give tiles of nearly one length.
 // Returns zc and the efficiency of the best zc + 2 count (steps of useful plane
 // work per resident slot over steps taken, 1 = perfect).
+static int box_zc(int nz, int zc)
+{
+    const int m = (nz + zc - 1) / zc;
+    return (nz + m - 1) / m;
+}
+
 template <class T>
-static int choose_zc(const std::vector<Box<T>> &boxes, long long slots, bool tma, double *score)
+static int choose_zc(const std::vector<Box<T>> &boxes, long long slots, bool tma, int width,
+                     double *score, double *steps)
 {
     int maxnz = 1;
     double planes = 0.0;  // tile-planes of useful work
     for (const auto &B : boxes) {
         maxnz = std::max(maxnz, B.nz);
-        planes += (double)tiles_of(TK_SWEEP, B.nx, B.ny, B.nz, B.nz) * B.nz;
+        planes += (double)tiles_of(TK_SWEEP, B.nx, B.ny, B.nz, B.nz, kColZ, width) * B.nz;
     }
     int best = std::min(kSweepZ, maxnz);
     double best_cost = -1.0, plain_cost = -1.0;
@@ -382,9 +397,15 @@ static int choose_zc(const std::vector<Box<T>> &boxes, long long slots, bool tma
         if (Z == last) continue;
         last = Z;
         long long ctas = 0;
-        for (const auto &B : boxes) ctas += tiles_of(TK_SWEEP, B.nx, B.ny, B.nz, Z);
+        int longest = 1;
+        for (const auto &B : boxes) {
+            const int zb = box_zc(B.nz, Z);
+            ctas += tiles_of(TK_SWEEP, B.nx, B.ny, B.nz, zb, kColZ, width);
+            longest = std::max(longest, zb);
+        }
         const long long waves = (ctas + slots - 1) / slots;
-        const double plain = (double)waves * (Z + 2), cost = (double)waves * (Z + (tma ? 4 : 2));
+        const double plain = (double)waves * (longest + 2),
+                     cost = (double)waves * (longest + (tma ? 4 : 2));
         if (plain_cost < 0.0 || plain < plain_cost) plain_cost = plain;
         if (best_cost < 0.0 || cost < best_cost - 1e-9) {
             best_cost = cost;
@@ -392,6 +413,7 @@ static int choose_zc(const std::vector<Box<T>> &boxes, long long slots, bool tma
         }
     }
     *score = planes / ((double)slots * plain_cost);
+    *steps = best_cost;
     return best;
 }
 
@@ -487,20 +509,20 @@ static int tail_cluster(int nbox)
 // levels of that size cost their loads of the weights instead.
 static bool tail_worth(long long cells, int cl) { return cells <= 3400LL * cl; }
 
-// Tensor maps of every box of an FP32 level set (TMA sweep); false if the
-// driver cannot encode them.
-// TMA maps of a level's boxes; *prol: they also hold each box's coarse phi
-// (the fused prolongation), which every box's coarse level must allow.
+// TMA maps of an FP32 level's boxes, false if the driver cannot encode them;
+// *prol: they also hold each box's coarse phi (the fused prolongation).  A
+// copy box may be larger than a box of the level: what lies outside its arrays
+// reads as zero, like the guards.  64 boxes of 32 to 128 cells a side (2.7e7
+// cells): 165 us a sweep fed by the TMA, 229 us with plain loads.
 template <class T>
-static bool plan_maps(const std::vector<Box<T>> &set, DescBlob &blob, size_t *off, bool *prol)
+static bool plan_maps(const std::vector<Box<T>> &set, int width, DescBlob &blob, size_t *off,
+                      bool *prol)
 {
     *prol = false;
     if (sizeof(T) != sizeof(float)) return false;
     bool cp = true;
     for (const Box<T> &B : set) {
-        if (!sweep_tma_fits(B.nx, B.ny)) return false;
-        cp = cp && B.phic && sweep_tma_prol_fits(B.nx, B.ny, B.nx / 2, B.ny / 2) &&
-             B.nz % 2 == 0;
+        cp = cp && B.phic && B.nx % 2 == 0 && B.ny % 2 == 0 && B.nz % 2 == 0;
     }
     const size_t one = sweep_maps_size();
     std::vector<char> bytes(one * set.size() + 128);   // tensor maps are 128-byte aligned
@@ -512,7 +534,7 @@ static bool plan_maps(const std::vector<Box<T>> &set, DescBlob &blob, size_t *of
         const float *pc = cp ? reinterpret_cast<const float *>(B.phic - B.cQ) : nullptr;
         if (!encode_sweep_maps(reinterpret_cast<SweepMaps *>(base + i * one), B.nx, B.ny, B.nz,
                                lb(B.phi), lb(B.phi2), lb(B.f), lb(B.wx), lb(B.wy), lb(B.wz), pc,
-                               B.nx / 2, B.ny / 2, B.nz / 2))
+                               B.nx / 2, B.ny / 2, B.nz / 2, width))
             return false;
     }
     *off = blob.put(base, one * set.size(), 128);
@@ -574,14 +596,27 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
         for (int b = 0; b < s->nbox; ++b)
             if (l < H.lc[b]) set.push_back(make_box(s, H, b, l));
         if (!set.empty()) {
-            double score = 0.0;
-            int zc = choose_zc(set, slots, tma, &score);
+            double score = 0.0, steps = 0.0;
+            int zc = choose_zc(set, slots, tma, 64, &score, &steps);
+            // the TMA sweep's tiles may also be 32 x 16: they leave fewer lanes
+            // idle where 64 does not divide a side (160 x 96 x 224: 30.5 -> 21.5
+            // us, 19 boxes of 96^3: 138 -> 91), and cost 3% more where it does
+            // (512^3: 556 -> 571 us), whose step counts are equal
+            int width = 64;
+            if (tma) {
+                double score32 = 0.0, steps32 = 0.0;
+                const int zc32 = choose_zc(set, slots, tma, 32, &score32, &steps32);
+                if (steps32 < steps) {
+                    width = 32;
+                    zc = zc32;
+                }
+            }
             if (s->opts.sweep_zc > 0) {   // the tile depth given (autotuned) instead
                 int maxnz = 1;
                 for (const auto &B : set) maxnz = std::max(maxnz, B.nz);
                 zc = std::min(s->opts.sweep_zc, maxnz);
             }
-            for (auto &B : set) B.zc = zc;
+            for (auto &B : set) B.zc = s->opts.sweep_zc > 0 ? zc : box_zc(B.nz, zc);
             // fused sweeps when the grid can keep the GPU busy, and only in
             // FP32: FP64 smoothing is bound by the FP64 pipe, where the red
             // ring the fused sweep recomputes costs more than the DRAM
@@ -595,9 +630,10 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
                          (s->opts.smoother == 2 || (s->opts.smoother == 0 && ok));
             size_t moff = 0;
             bool prol = false;
-            if (H.fused[l] && tma && s->tma && plan_maps(set, blob, &moff, &prol)) {
+            if (H.fused[l] && tma && s->tma && plan_maps(set, width, blob, &moff, &prol)) {
                 map_offs->push_back({l, moff});  // else: plain-load sweeps on this level
                 H.prol[l] = prol ? 1 : 0;
+                for (auto &B : set) B.sw = width;
             }
         }
         // the level below, where it smooths with passes, takes its first red

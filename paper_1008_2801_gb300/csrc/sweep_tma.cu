@@ -2,7 +2,7 @@
 // Accelerator, warp-specialised (sm_103a).
 //
 // Same schedule and arithmetic as k_rbgs_sweep (kernels.cu), and bitwise the
-// same result: a CTA owns a 64 x 8 tile and a chunk of planes, marches
+// same result: a CTA owns a 64 x 8 (or 32 x 16) tile and a chunk of planes, marches
 // upward, computes the new red values of plane k (its tile plus a one-cell
 // ring) and the new black values of plane k-1, out of place.  The roles are
 // split over warps:
@@ -36,7 +36,7 @@
 // the named barrier); the producer stops issuing, and before it exits it
 // waits, with the default bound, for every copy it issued.
 //
-// TMA rules kept: every copy starts at x = x0 - 4 (x0 a multiple of 64), a
+// TMA rules kept: every copy starts at x = x0 - 4 (x0 a multiple of 32), a
 // multiple of 4 floats = 16 bytes; rows are P floats with P a multiple of 8;
 // shared destinations are 128-byte aligned; only loads use out-of-range
 // (negative) coordinates, which read zeros.
@@ -51,40 +51,44 @@ namespace mg {
 
 namespace {
 
-constexpr int kTileW = 72;                 // x0 - 4 .. x0 + 67
-constexpr int kSrcRows = kSweepTY + 4;     // y0 - 2 .. y0 + 9
-constexpr int kOpRows = kSweepTY + 2;      // y0 - 1 .. y0 + 8
-constexpr int kWyRows = kSweepTY + 3;      // y0 - 1 .. y0 + 9 (faces)
-constexpr int kConsumers = kSweepTY + 3;   // row warps, 2 ring-row warps, 1 ring-column warp
+constexpr int kConsumers = kSweepTY + 3;   // 8 row warps, 2 ring-row warps, 1 ring-column warp
 constexpr int kTmaThreads = 32 * (kConsumers + 1);
 
 constexpr int pad128(int bytes) { return (bytes + 127) / 128 * 128; }
-constexpr int kSrcBytes = kSrcRows * kTileW * 4;
-constexpr int kOpBytes = kOpRows * kTileW * 4;
-constexpr int kWyBytes = kWyRows * kTileW * 4;
-constexpr int kSrcOff = 0;
-constexpr int kFOff = kSrcOff + pad128(kSrcBytes);
-constexpr int kWxOff = kFOff + pad128(kOpBytes);
-constexpr int kWyOff = kWxOff + pad128(kOpBytes);
-constexpr int kWzOff = kWyOff + pad128(kWyBytes);
-constexpr int kStageBytes = kWzOff + pad128(kOpBytes);
-constexpr unsigned kTxBytes = kSrcBytes + 3 * kOpBytes + kWyBytes;  // bytes landing per stage
-// With the prolongation fused (the first post-smoothing sweep): the coarse
-// correction under the phi tile, coarse columns x0/2 - 4 .. x0/2 + 35 and
-// rows y0/2 - 1 .. y0/2 + 4 of coarse plane p/2, after the stage's regions
-constexpr int kEcW = 40, kEcRows = kSweepTY / 2 + 2;
-constexpr int kEcOff = kStageBytes;
-constexpr int kEcBytes = kEcW * kEcRows * 4;
-constexpr int kStageBytesP = kEcOff + pad128(kEcBytes);
-constexpr int kRedSW = 2 * kTX + 2, kRedPlane = (kSweepTY + 2) * kRedSW;   // red ring, floats
-
 // Two red planes: a step writes plane k's and reads plane k-1's, and ends at a
 // barrier.
 constexpr int kRedPlanes = 2;
-constexpr int smem_bytes(int ns, bool prol = false)
-{
-    return ns * (prol ? kStageBytesP : kStageBytes) + pad128(kRedPlanes * kRedPlane * 4) + 128;
-}
+
+// A tile W cells wide and TY high (512 cells), and the staged copies under it.
+template <int W>
+struct Geo {
+    static constexpr int TY = 512 / W;              // rows
+    static constexpr int LP = W / 2;                // lanes (pairs) of a row
+    static constexpr int TW = W + 8;                // staged columns x0 - 4 .. x0 + W + 3
+    static constexpr int SrcRows = TY + 4;          // y0 - 2 .. y0 + TY + 1
+    static constexpr int OpRows = TY + 2;           // y0 - 1 .. y0 + TY
+    static constexpr int WyRows = TY + 3;           // y0 - 1 .. y0 + TY + 1 (faces)
+    static constexpr int SrcBytes = SrcRows * TW * 4;
+    static constexpr int OpBytes = OpRows * TW * 4;
+    static constexpr int WyBytes = WyRows * TW * 4;
+    static constexpr int FOff = pad128(SrcBytes);   // phi at 0
+    static constexpr int WxOff = FOff + pad128(OpBytes);
+    static constexpr int WyOff = WxOff + pad128(OpBytes);
+    static constexpr int WzOff = WyOff + pad128(WyBytes);
+    static constexpr unsigned TxBytes = SrcBytes + 3 * OpBytes + WyBytes;  // bytes landing per stage
+    // With the prolongation fused (the first post-smoothing sweep): the coarse
+    // correction under the phi tile, coarse columns x0/2 - 4 .. x0/2 + W/2 + 3
+    // and rows y0/2 - 1 .. y0/2 + TY/2 of coarse plane p/2
+    static constexpr int EcW = W / 2 + 8, EcRows = TY / 2 + 2;
+    static constexpr int EcOff = WzOff + pad128(OpBytes);
+    static constexpr int EcBytes = EcW * EcRows * 4;
+    static constexpr int RedSW = W + 2, RedPlane = (TY + 2) * RedSW;   // a red plane, floats
+    __host__ __device__ static constexpr int stage_bytes(bool prol) { return EcOff + (prol ? pad128(EcBytes) : 0); }
+    __host__ __device__ static constexpr int smem_bytes(int ns, bool prol)
+    {
+        return ns * stage_bytes(prol) + pad128(kRedPlanes * RedPlane * 4) + 128;
+    }
+};
 
 // the configuration the library launches: 6 stages, 2 CTAs (24 warps) per SM
 constexpr int kStages = 6, kMinCtas = 2;
@@ -195,10 +199,11 @@ struct Ring {
     }
 };
 
-// Element of the staged coarse tile (40 x 6 cells) under column (x, y).
+// Element of the staged coarse tile under column (x, y).
+template <int W>
 __device__ __forceinline__ int coarse_at(int x, int y, int x0, int y0)
 {
-    return kEcOff / 4 + ((y >> 1) - (y0 >> 1) + 1) * kEcW + (x >> 1) - (x0 >> 1) + 4;
+    return Geo<W>::EcOff / 4 + ((y >> 1) - (y0 >> 1) + 1) * Geo<W>::EcW + (x >> 1) - (x0 >> 1) + 4;
 }
 
 // PROL: the level's prolongation phi += e(parent) (the coarse correction,
@@ -209,16 +214,17 @@ __device__ __forceinline__ int coarse_at(int x, int y, int x0, int y0)
 // neighbours and a black update only the new red values, so the sweep's
 // result is bitwise that of prolongation then sweep; the level's phi in
 // memory stays unprolonged, which the out-of-place sweep never reads again.
-template <int NS, int MINB, bool PROL>
+template <int W, int NS, int MINB, bool PROL>
 __global__ void __launch_bounds__(kTmaThreads, MINB)
     k_rbgs_sweep_tma(BoxSet<float> S, const SweepMaps *__restrict__ maps,
                      const int *__restrict__ active, int src_is_phi2, int *__restrict__ err,
                      long long polls)
 {
-    constexpr int STG = (PROL ? kStageBytesP : kStageBytes) / 4;   // stage stride, floats
+    using G = Geo<W>;
+    constexpr int STG = G::stage_bytes(PROL) / 4;   // stage stride, floats
     static_assert(NS >= 3, "planes k and k + 1 are held, another is in flight");
-    constexpr int PHI = kSrcOff / 4, FF = kFOff / 4, WX = kWxOff / 4, WY = kWyOff / 4,
-                  WZ = kWzOff / 4, TW = kTileW, SW = kRedSW;
+    constexpr int PHI = 0, FF = G::FOff / 4, WX = G::WxOff / 4, WY = G::WyOff / 4,
+                  WZ = G::WzOff / 4, TW = G::TW, SW = G::RedSW, TY = G::TY, LP = G::LP;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
@@ -228,8 +234,8 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
 
     const int *ts = S.tstart[TK_SWEEP];
     const int ntile = S.ntiles[TK_SWEEP];
-    // tile t of the plain sweep's index space (2D tiles of 32 pairs x 8 rows);
-    // the box it belongs to is skipped when it is not active
+    // tile t of the set's TK_SWEEP index space; the box it belongs to is skipped
+    // when it is not active
     struct Tile {
         int b, x0, y0, z0, z1;
         bool on;
@@ -238,13 +244,11 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
         Tile T;
         T.b = find_box(ts, S.nbox, t);
         const Box<float> &B = S.boxes[T.b];
-        int ex, ey, ez;
-        tile_extent(TK_SWEEP, B.nx, B.ny, B.nz, ex, ey, ez, B.zc);
-        const int ntx = (ex + kTX - 1) / kTX, nty = (ey + kSweepTY - 1) / kSweepTY;
+        const int ntx = (B.nx + W - 1) / W, nty = (B.ny + TY - 1) / TY;
         int loc = t - ts[T.b];
-        T.x0 = loc % ntx * 2 * kTX;
+        T.x0 = loc % ntx * W;
         loc /= ntx;
-        T.y0 = loc % nty * kSweepTY;
+        T.y0 = loc % nty * TY;
         T.z0 = loc / nty * B.zc;
         T.z1 = min(T.z0 + B.zc, B.nz);
         T.on = !active || active[B.box];
@@ -266,20 +270,35 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
         // from the NS-th on it waits until the consumers have released the
         // stage.  It runs on into the next tile while they finish this one.
         if (lane == 0) {
-            int i = 0, mapped = -1;
+            int i = 0;
             bool ok = true;
-            for (int t = blockIdx.x; ok && t < ntile; t += gridDim.x) {
-                const Tile T = tile_at(t);
-                if (!T.on) continue;
-                const SweepMaps &M = maps[T.b];
-                if (T.b != mapped) {
-                    for (int m = 0; m < (PROL ? 7 : 6); ++m) tensormap_acquire(&M.m[m]);
-                    mapped = T.b;
+            // the next tile of an active box
+            auto next_tile = [&](int t, Tile &T) {
+                for (; t < ntile; t += gridDim.x) {
+                    T = tile_at(t);
+                    if (T.on) break;
                 }
+                return t;
+            };
+            auto acquire = [&](int b) {
+                for (int m = 0; m < (PROL ? 7 : 6); ++m) tensormap_acquire(&maps[b].m[m]);
+            };
+            Tile T, N;
+            int t = next_tile(blockIdx.x, T), tn = t;
+            if (t < ntile) acquire(T.b);
+            for (; ok && t < ntile; t = tn, T = N) {
+                const SweepMaps &M = maps[T.b];
+                tn = -1;
                 const CUtensorMap *msrc = &M.m[src_is_phi2 ? 1 : 0];
                 const int x0 = T.x0, y0 = T.y0;
                 for (int p = T.z0 - 2; p <= T.z1 + 1; ++p, ++i) {
                     const int s = i % NS;
+                    if (p == min(T.z0 + NS - 2, T.z1 + 1)) {
+                        // a ring of planes is in flight: look the next tile up
+                        // and acquire its box's maps meanwhile
+                        tn = next_tile(t + gridDim.x, N);
+                        if (tn < ntile && N.b != T.b) acquire(N.b);
+                    }
                     if (i >= NS &&
                         !mbar_wait(smem_addr(&empty[s]), (unsigned)(((i / NS) - 1) & 1), polls)) {
                         atomicExch(err, 1);
@@ -288,17 +307,17 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
                     }
                     unsigned char *base = smem + s * (STG * 4);
                     const unsigned bar = smem_addr(&full[s]);
-                    mbar_expect_tx(bar, kTxBytes + (PROL ? kEcBytes : 0));
+                    mbar_expect_tx(bar, G::TxBytes + (PROL ? G::EcBytes : 0));
                     const int zt = p + 1;  // tensor z of logical plane p (guard plane first)
-                    tma_load_3d(smem_addr(base + kSrcOff), msrc, bar, x0 - 4, y0 - 2, zt);
-                    tma_load_3d(smem_addr(base + kFOff), &M.m[2], bar, x0 - 4, y0 - 1, zt);
-                    tma_load_3d(smem_addr(base + kWxOff), &M.m[3], bar, x0 - 4, y0 - 1, zt);
-                    tma_load_3d(smem_addr(base + kWyOff), &M.m[4], bar, x0 - 4, y0 - 1, zt);
-                    tma_load_3d(smem_addr(base + kWzOff), &M.m[5], bar, x0 - 4, y0 - 1, zt);
+                    tma_load_3d(smem_addr(base), msrc, bar, x0 - 4, y0 - 2, zt);
+                    tma_load_3d(smem_addr(base + G::FOff), &M.m[2], bar, x0 - 4, y0 - 1, zt);
+                    tma_load_3d(smem_addr(base + G::WxOff), &M.m[3], bar, x0 - 4, y0 - 1, zt);
+                    tma_load_3d(smem_addr(base + G::WyOff), &M.m[4], bar, x0 - 4, y0 - 1, zt);
+                    tma_load_3d(smem_addr(base + G::WzOff), &M.m[5], bar, x0 - 4, y0 - 1, zt);
                     // the coarse correction under plane p: coarse plane p >> 1
                     // (planes -1, -2: the coarse guard plane, zero)
                     if (PROL)
-                        tma_load_3d(smem_addr(base + kEcOff), &M.m[6], bar, x0 / 2 - 4,
+                        tma_load_3d(smem_addr(base + G::EcOff), &M.m[6], bar, x0 / 2 - 4,
                                     y0 / 2 - 1, (p >> 1) + 1);
                 }
             }
@@ -312,7 +331,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
     }
 
     // consumers
-    const int cw = warp - 1;           // 0..7 row warps, 8 / 9 ring rows, 10 ring column
+    const int cw = warp - 1;   // 0..7 row warps, 8 / 9 ring rows, 10 ring column
     Ring<NS> rg;
     long long left = polls;
     auto take = [&]() {   // the next plane's stage, once the plane has landed in it
@@ -331,29 +350,33 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
     int r0 = 0;   // where the current plane's red values go
 
     if (cw < kSweepTY + 2) {
-        // Rows y0 - 1 .. y0 + 8: lane owns the pair (xa, xa + 1), whose red cell
-        // on plane k is at position q = (y + k) & 1.  A row's q is uniform and
-        // the planes alternate, so the loop holds a step for either q, with
+        // Rows y0 - 1 .. y0 + TY: lane owns the pair (xa, xa + 1), whose red cell
+        // on plane k is at position q = (y + k) & 1.  A warp takes one row of 32
+        // pairs, or rows r and r + 2 of 16, so q is uniform; the planes
+        // alternate, so the loop holds a step for either q, with
         // every position a constant (unrolled over the stages as well, the row
         // kinds and parities made 30 step bodies, and the warps waited for
         // instructions).
         auto march = [&](auto own_tag) {
             constexpr bool OWN = decltype(own_tag)::value;   // row of the tile: black cells too
-            const int row = OWN ? cw + 1 : cw == kSweepTY ? 0 : kSweepTY + 1;   // 0 .. 9
-            const int pa = (row + 1) * TW + 2 * lane + 4;    // phi region, of xa
-            const int oa = row * TW + 2 * lane + 4;          // operand regions
-            const int ra = row * SW + 2 * lane + 1;          // red plane
+            const int lp = lane % LP;
+            const int row = !OWN ? (cw == kSweepTY ? 0 : TY + 1)                // 0 .. TY + 1
+                            : LP == 32 ? cw + 1 : (cw >> 1) * 4 + (cw & 1) + 2 * (lane / LP) + 1;
+            const bool lane_on = OWN || lane < LP;           // (a ring row is one row)
+            const int pa = (row + 1) * TW + 2 * lp + 4;      // phi region, of xa
+            const int oa = row * TW + 2 * lp + 4;            // operand regions
+            const int ra = row * SW + 2 * lp + 1;            // red plane
             for (int t = blockIdx.x; t < ntile; t += gridDim.x) {
             const Tile T = tile_at(t);
             if (!T.on) continue;
             const Box<float> &B = S.boxes[T.b];
             const int nx = B.nx, ny = B.ny, nz = B.nz, z0 = T.z0, z1 = T.z1;
             const long long Q = B.Q;
-            const int y = T.y0 + row - 1, xa = T.x0 + 2 * lane;
+            const int y = T.y0 + row - 1, xa = T.x0 + 2 * lp;
             const bool vy = y >= 0 && y < ny;
             const bool v0 = vy && xa < nx, v1 = vy && xa + 1 < nx;
-            const int ec = coarse_at(xa, y, T.x0, T.y0), es = coarse_at(xa, y - 1, T.x0, T.y0),
-                      en = coarse_at(xa, y + 1, T.x0, T.y0);
+            const int ec = coarse_at<W>(xa, y, T.x0, T.y0), es = coarse_at<W>(xa, y - 1, T.x0, T.y0),
+                      en = coarse_at<W>(xa, y + 1, T.x0, T.y0);
             const bool orow = OWN && y < ny;
             float *gdst = (src_is_phi2 ? B.phi : B.phi2) + (long long)(z0 - 2) * Q +
                           (long long)y * B.P + xa;           // plane k - 1
@@ -381,7 +404,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
                 const int sP = take();
                 const float *const S0 = sm + s0 * STG, *const SP = sm + sP * STG;
                 float *const R0 = red + r0;
-                const float *const R1 = red + (kRedPlane - r0);
+                const float *const R1 = red + (G::RedPlane - r0);
                 // operands of plane k (the red cell's now, the black cell's on
                 // the next step) and the black value above
                 float up = SP[PHI + pa + q], outer = S0[PHI + pa + (q ? 2 : -1)],
@@ -435,7 +458,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
                 float val = red_update(q ? be : outer, q ? outer : be, so, no, dn, up, x0w, x1w,
                                        y0w, y1w, z0w, z1w, fR);
                 val = (q ? v1 : v0) && k >= 0 && k < nz ? val : 0.f;
-                R0[ra + q] = val;
+                if (lane_on) R0[ra + q] = val;
                 // (2) the black value of plane k - 1, at the same position: its
                 // neighbour in the pair and those above and below are this
                 // thread's own red values
@@ -468,7 +491,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
                 wz = wzn;
                 named_barrier(1, 32 * kConsumers);
                 s0 = sP;
-                r0 = kRedPlane - r0;
+                r0 = G::RedPlane - r0;
                 gdst += Q;
                 ++k;
             };
@@ -490,10 +513,10 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
         return;
     }
 
-    // the ring columns x0 - 1 (lanes 0..3) and x0 + 64 (lanes 4..7): a lane owns
-    // the pair (yy, yy + 1), red at position q = (xc + y0 + k) & 1
-    const bool on = lane < kSweepTY;
-    const int cx = lane < kSweepTY / 2 ? -1 : 2 * kTX, cy = 2 * (lane % (kSweepTY / 2));
+    // the ring columns x0 - 1 (the first TY / 2 lanes) and x0 + W (the next): a
+    // lane owns the pair (yy, yy + 1), red at position q = (xc + y0 + k) & 1
+    const bool on = lane < TY;
+    const int cx = lane < TY / 2 ? -1 : W, cy = 2 * (lane % (TY / 2));
     const int pc = (cy + 2) * TW + cx + 4, oc = pc - TW, rc = (cy + 1) * SW + cx + 1;
     for (int t = blockIdx.x; t < ntile; t += gridDim.x) {
         const Tile T = tile_at(t);
@@ -504,8 +527,8 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
         const bool vx = on && xc >= 0 && xc < B.nx;
         const bool v0 = vx && yy < B.ny, v1 = vx && yy + 1 < B.ny;
         // (the parents of a pair's rows are one row of the coarse tile)
-        const int ec = coarse_at(xc, yy, T.x0, T.y0), ew = coarse_at(xc - 1, yy, T.x0, T.y0),
-                  ee = coarse_at(xc + 1, yy, T.x0, T.y0);
+        const int ec = coarse_at<W>(xc, yy, T.x0, T.y0), ew = coarse_at<W>(xc - 1, yy, T.x0, T.y0),
+                  ee = coarse_at<W>(xc + 1, yy, T.x0, T.y0);
         int q = (xc + T.y0 + z0 - 1) & 1;
         const int sA = take();
         int s0 = take();
@@ -534,7 +557,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
                     if (PROL) {
                         we += S0[ew];
                         ea += S0[ee];
-                        out += S0[ec + (q ? kEcW : -kEcW)];
+                        out += S0[ec + (q ? G::EcW : -G::EcW)];
                     }
                     const float val =
                         red_update(we, ea, q ? be : out, q ? out : be, dn, up, S0[WX + o],
@@ -549,7 +572,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
             release(s0);
             named_barrier(1, 32 * kConsumers);
             s0 = sP;
-            r0 = kRedPlane - r0;
+            r0 = G::RedPlane - r0;
         }
         release(s0);   // plane z1 + 1
     }
@@ -578,18 +601,15 @@ EncodeTiledFn encoder()
 
 }  // namespace
 
-// Encode the maps of a box level (arrays given by their allocation base =
-// logical (0, 0, -1)): phi, phi2, f, wx, wy, wz, and with phic_base the
-// coarse level's phi (cx x cy x cz cells) for the fused prolongation.
-// Returns false if the driver cannot (or a box does not fit).
-bool encode_sweep_maps(SweepMaps *out, int nx, int ny, int nz, const float *phi_base,
-                       const float *phi2_base, const float *f_base, const float *wx_base,
-                       const float *wy_base, const float *wz_base, const float *phic_base,
-                       int cx, int cy, int cz)
+template <int W>
+static bool encode_maps(SweepMaps *out, int nx, int ny, int nz, const float *phi_base,
+                        const float *phi2_base, const float *f_base, const float *wx_base,
+                        const float *wy_base, const float *wz_base, const float *phic_base,
+                        int cx, int cy, int cz)
 {
+    using G = Geo<W>;
     EncodeTiledFn fn = encoder();
     if (!fn) return false;
-    if (!sweep_tma_fits(nx, ny)) return false;
     const cuuint32_t ones[3] = {1, 1, 1};
     auto enc = [&](CUtensorMap *m, const float *base, int mx, int my, int mz,
                    const cuuint32_t *box) {
@@ -601,27 +621,43 @@ bool encode_sweep_maps(SweepMaps *out, int nx, int ny, int nz, const float *phi_
                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
-    const cuuint32_t box_src[3] = {kTileW, kSrcRows, 1};
-    const cuuint32_t box_op[3] = {kTileW, kOpRows, 1};
-    const cuuint32_t box_wy[3] = {kTileW, kWyRows, 1};
+    const cuuint32_t box_src[3] = {G::TW, G::SrcRows, 1};
+    const cuuint32_t box_op[3] = {G::TW, G::OpRows, 1};
+    const cuuint32_t box_wy[3] = {G::TW, G::WyRows, 1};
     const float *base[6] = {phi_base, phi2_base, f_base, wx_base, wy_base, wz_base};
     const cuuint32_t *box[6] = {box_src, box_src, box_op, box_op, box_wy, box_op};
     for (int i = 0; i < 6; ++i)
         if (!enc(&out->m[i], base[i], nx, ny, nz, box[i])) return false;
     memset(&out->m[6], 0, sizeof(CUtensorMap));
     if (phic_base) {
-        if (!sweep_tma_prol_fits(nx, ny, cx, cy)) return false;
-        const cuuint32_t box_ec[3] = {kEcW, kEcRows, 1};
+        if (nx != 2 * cx || ny != 2 * cy) return false;
+        const cuuint32_t box_ec[3] = {G::EcW, G::EcRows, 1};
         if (!enc(&out->m[6], phic_base, cx, cy, cz, box_ec)) return false;
     }
     return true;
 }
 
-// The fused prolongation reads a 40 x 6 coarse tile: the coarse rows and
-// planes hold it, and the level is twice the coarse one in x and y.
+// Encode the maps of a box level (arrays given by their allocation base =
+// logical (0, 0, -1)): phi, phi2, f, wx, wy, wz, and with phic_base the
+// coarse level's phi (cx x cy x cz cells) for the fused prolongation; width: of
+// the tiles (64 or 32).
+// Returns false if the driver cannot.
+bool encode_sweep_maps(SweepMaps *out, int nx, int ny, int nz, const float *phi_base,
+                       const float *phi2_base, const float *f_base, const float *wx_base,
+                       const float *wy_base, const float *wz_base, const float *phic_base,
+                       int cx, int cy, int cz, int width)
+{
+    return width == 32 ? encode_maps<32>(out, nx, ny, nz, phi_base, phi2_base, f_base, wx_base,
+                                         wy_base, wz_base, phic_base, cx, cy, cz)
+                       : encode_maps<64>(out, nx, ny, nz, phi_base, phi2_base, f_base, wx_base,
+                                         wy_base, wz_base, phic_base, cx, cy, cz);
+}
+
+// The single-stage entry points take the fused prolongation only where the
+// coarse rows and planes hold a whole 40 x 6 tile.
 bool sweep_tma_prol_fits(int nx, int ny, int cx, int cy)
 {
-    return nx == 2 * cx && ny == 2 * cy && pitch_row(cx) >= kEcW && cy + 1 >= kEcRows;
+    return nx == 2 * cx && ny == 2 * cy && pitch_row(cx) >= Geo<64>::EcW && cy + 1 >= Geo<64>::EcRows;
 }
 
 size_t sweep_maps_size() { return sizeof(SweepMaps); }
@@ -630,7 +666,7 @@ size_t sweep_maps_size() { return sizeof(SweepMaps); }
 // that two CTAs fit on an SM.  Function attributes are per device: they
 // are set once on each device, the first time a launch or an occupancy
 // query runs with that device current.
-template <int NS, int MINB, bool PROL>
+template <int W, int NS, int MINB, bool PROL>
 static void set_smem_attributes()
 {
     constexpr int kMaxDevices = 64;
@@ -643,24 +679,25 @@ static void set_smem_attributes()
     }
     std::lock_guard<std::mutex> lk(mu);
     if (dev >= 0 && done[dev]) return;
-    cudaFuncSetAttribute(k_rbgs_sweep_tma<NS, MINB, PROL>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(NS, PROL));
-    cudaFuncSetAttribute(k_rbgs_sweep_tma<NS, MINB, PROL>,
+    cudaFuncSetAttribute(k_rbgs_sweep_tma<W, NS, MINB, PROL>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         Geo<W>::smem_bytes(NS, PROL));
+    cudaFuncSetAttribute(k_rbgs_sweep_tma<W, NS, MINB, PROL>,
                          cudaFuncAttributePreferredSharedMemoryCarveout,
                          cudaSharedmemCarveoutMaxShared);
     if (dev >= 0) done[dev] = true;
 }
 
-// Levels whose rows and planes hold a whole copy box (72 x 12).
-bool sweep_tma_fits(int nx, int ny) { return pitch_row(nx) >= kTileW && ny + 1 >= kSrcRows; }
+// (They also ask for rows and planes that hold a whole 72 x 12 copy box.)
+bool sweep_tma_fits(int nx, int ny) { return pitch_row(nx) >= Geo<64>::TW && ny + 1 >= Geo<64>::SrcRows; }
 
 int sweep_tma_ctas_per_sm()
 {
     int n = 0;
-    set_smem_attributes<kStages, kMinCtas, false>();
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rbgs_sweep_tma<kStages, kMinCtas, false>,
+    set_smem_attributes<64, kStages, kMinCtas, false>();
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_rbgs_sweep_tma<64, kStages, kMinCtas, false>,
                                                       kTmaThreads,
-                                                      smem_bytes(kStages)) != cudaSuccess) {
+                                                      Geo<64>::smem_bytes(kStages, false)) != cudaSuccess) {
         cudaGetLastError();
         return 1;
     }
@@ -699,21 +736,24 @@ cudaError_t launch_rbgs_sweep_tma(const BoxSet<float> &S, const SweepMaps *maps,
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(std::min(S.ntiles[TK_SWEEP], resident_ctas()));
     cfg.blockDim = dim3(kTmaThreads);
-    cfg.dynamicSmemBytes = smem_bytes(kStages, prolong);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl_enabled() ? 1 : 0;
-    if (prolong) {
-        set_smem_attributes<kStages, kMinCtas, true>();
-        return cudaLaunchKernelEx(&cfg, k_rbgs_sweep_tma<kStages, kMinCtas, true>, S, maps, active,
-                                  src_is_phi2, err, wait_polls);
-    }
-    set_smem_attributes<kStages, kMinCtas, false>();
-    return cudaLaunchKernelEx(&cfg, k_rbgs_sweep_tma<kStages, kMinCtas, false>, S, maps, active,
-                              src_is_phi2, err, wait_polls);
+    auto go = [&](auto width, auto prol) {
+        constexpr int W = decltype(width)::value;
+        constexpr bool PR = decltype(prol)::value;
+        set_smem_attributes<W, kStages, kMinCtas, PR>();
+        cfg.dynamicSmemBytes = Geo<W>::smem_bytes(kStages, PR);
+        return cudaLaunchKernelEx(&cfg, k_rbgs_sweep_tma<W, kStages, kMinCtas, PR>, S, maps,
+                                  active, src_is_phi2, err, wait_polls);
+    };
+    const std::integral_constant<int, 64> w64;
+    const std::integral_constant<int, 32> w32;
+    if (S.sweep_w == 32) return prolong ? go(w32, std::true_type{}) : go(w32, std::false_type{});
+    return prolong ? go(w64, std::true_type{}) : go(w64, std::false_type{});
 }
 
 }  // namespace mg
