@@ -1158,29 +1158,46 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         const int l = down ? step : 2 * (nl - 1) - step;
         const bool split = l < nd;
         if (!down && l == nd - 1) cl.sync();   // the first CTA's correction is there
-        if (!split && rank != 0) continue;
         const TailView<T> V = views[l];
-        auto sync = [&]() {
-            if (split) cl.sync();
-            else __syncthreads();
-        };
-        if (l == nl - 1) {   // the coarsest level: phi = A^{-1} f, a warp per row
+        if (l == nl - 1) {
+            // the coarsest level: phi = A^{-1} f, a warp per row.  A large
+            // inverse is read by every CTA of the cluster (567 cells in FP64
+            // on one SM's pipe: 77 us), a part of the rows each.
             const Box<T> &B = J.lv[l];
             const int n = V.nx * V.ny * B.nz;
+            const bool shared = CL > 1 && J.ainv < 0;
+            if (!shared && rank != 0) continue;
+            T *phi = V.phi;
+            if (shared) {
+                cl.sync();   // the first CTA's f is there
+                if (rank != 0) {
+                    const T *const f0 = cl.map_shared_rank(V.f, 0);
+                    for (int q = tid; q < n; q += kTailThreads) V.f[q] = f0[q];
+                    __syncthreads();
+                    phi = cl.map_shared_rank(V.phi, 0);
+                }
+            }
             const float rx = __frcp_rn((float)V.nx), ry = __frcp_rn((float)V.ny);
-            for (int r = warp; r < n; r += kTailThreads / 32) {
+            const int nw = kTailThreads / 32;
+            for (int r = shared ? rank * nw + warp : warp; r < n; r += shared ? CL * nw : nw) {
                 const T *row = (J.ainv >= 0 ? sm + J.ainv : B.ainv) + (long long)r * n;
                 T acc = T(0);
                 for (int q = lane; q < n; q += 32) acc = fmadd(row[q], V.f[q], acc);
                 for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
                 if (lane == 0) {
                     const int t = tail_div(r, rx), k = tail_div(t, ry);
-                    V.phi[tail_at(V, r - t * V.nx, t - k * V.ny, k)] = acc;
+                    phi[(k + 1) * V.q + (t - k * V.ny + 1) * V.p + r - t * V.nx + 1] = acc;
                 }
             }
-            __syncthreads();
+            if (shared) cl.sync();
+            else __syncthreads();
             continue;
         }
+        if (!split && rank != 0) continue;
+        auto sync = [&]() {
+            if (split) cl.sync();
+            else __syncthreads();
+        };
         const int nu = down ? nu1 : nu2, first = down ? 0 : post_first;
         const TailWalk W(V.nx >> 1, V.ny, V.np);
         if (!down) {
@@ -1814,58 +1831,71 @@ __device__ __forceinline__ void round_at(int nx, int ny, int nz, int P, long lon
     }
 }
 
-// The calling CTA assembles M = -A (symmetric positive definite) densely in
-// `a`, inverts it by Gauss-Jordan elimination without pivoting (M is
-// diagonally dominant, or symmetric positive definite after the shift below)
-// and writes A^{-1} = -M^{-1} (FP64, and FP32 if inv32).  When every wall is
-// Neumann (`singular`), M is only semi-definite with the constants as null
-// space; c 1 1^T with c = trace(M) / n^2 is added, which makes it positive
-// definite: applied to r it gives a solution of M x = r - mean(r) (the
-// constant part of r, which no solution can match, is dropped), and the
-// zero-mean one when r has zero mean.
-// Storage of the symmetric matrix M being inverted.  Only entries (i, j)
-// with i <= j are stored, written or read.  Full: row-major n x n (global
-// scratch, any n; the lower triangle is left alone).  Packed: the upper
-// triangle row by row, n (n + 1) / 2 entries (shared memory when it fits;
-// row i holds (i, i..n-1) from i n - i (i - 1) / 2 on).
-template <class R, bool PACKED>
-struct SymStore {
+// Dense inverses of the coarsest levels: M = -A (symmetric positive definite)
+// is assembled and inverted in place by Gauss-Jordan elimination without
+// pivoting (M is diagonally dominant, or positive definite after the shift
+// below), A^{-1} = -M^{-1}.  When every wall is Neumann (`singular`), M is only
+// semi-definite with the constants as null space; c 1 1^T with c = trace(M) /
+// n^2 is added, which makes it positive definite: applied to r it gives a
+// solution of M x = r - mean(r) (the constant part of r, which no solution can
+// match, is dropped), and the zero-mean one when r has zero mean.
+//
+// Only the upper triangle is kept: after pivots 0..p an entry with exactly one
+// index <= p is the negative of its mirror and every other entry equals its
+// mirror, so each pivot costs n^2/2 updates.  The rows are dealt out over the
+// CTAs of one cluster (row i to rank i % CTAs), in shared memory when they fit
+// (n <= 890 in FP64 on 16 CTAs), else in global scratch; a pivot needs its
+// column, which every owner stores into every CTA as it updates it, and one
+// cluster barrier.  What bounds it: n pivots of a barrier (~0.5 us) plus
+// n^2/2 FMAs on the FP64 pipes of 16 SMs.  A row's updates are those of a
+// single CTA in the same order, so the inverse is the same bit for bit.  One CTA
+// per box took 30.5 ms for 567 cells (FP64), 1.79 ms for the 192-cell boxes of
+// a batch, 181 us for 105 cells (FP32); these take 3.6 ms, 0.68 ms and 128 us.
+constexpr int kInvThreads = 512;
+
+// The rows of rank's part.  Row i = rank + ncta m holds (i, i..n-1).
+template <class R>
+struct InvRows {
     R *a;
-    int n;
-    __device__ __forceinline__ long long size() const
+    int n, rank, ncta;
+    bool packed;
+    __device__ __forceinline__ R *row(int m) const
     {
-        return PACKED ? (long long)n * (n + 1) / 2 : (long long)n * n;
+        const long long i = rank + (long long)ncta * m;
+        return a + (packed ? (long long)m * (n - rank) - (long long)ncta * m * (m - 1) / 2 : i * n + i);
     }
-    // entry (i, i); entry (i, j), j >= i, is row(i)[j - i]
-    __device__ __forceinline__ R *row(int i) const
+    // row i if it is this rank's, else NULL
+    __device__ __forceinline__ R *own(int i) const
     {
-        return a + (PACKED ? (long long)i * n - (long long)i * (i - 1) / 2 : (long long)i * n + i);
+        return i % ncta == rank ? row(i / ncta) : nullptr;
     }
-    __device__ __forceinline__ R &operator()(int i, int j) const { return row(i)[j - i]; }
+    __device__ __forceinline__ int count() const { return rank < n ? (n - 1 - rank) / ncta + 1 : 0; }
 };
 
-// Packed FP64 / FP32 matrices up to this size are inverted in shared memory
-// (n <= 225 in FP64, n <= 319 in FP32).
-constexpr int kPackedBottomBytes = 200 * 1024;
+__host__ __device__ inline long long inv_rows_elems(int n, int ncta)   // rank 0's, the most
+{
+    const long long m = (n - 1) / ncta + 1;
+    return m * n - (long long)ncta * m * (m - 1) / 2;
+}
 
-// The upper triangle of the block of M = -A of one box, rows and columns
-// from `at` on (the box's cells in C order): diagonal = sum of the six
-// weights, -w to each later neighbour inside the box (the earlier ones are
-// the mirrors).  Called by every thread of the CTA.
-template <class S, class W>
+// The block of M = -A of one box, rows and columns from `at` on (the box's
+// cells in C order): diagonal = sum of the six weights, -w to each later
+// neighbour inside the box (the earlier ones are the mirrors).
+template <class R, class W>
 __device__ __forceinline__ void assemble_box_block(int nx, int ny, int nz, int P, long long Q,
                                                    const W *__restrict__ wx,
                                                    const W *__restrict__ wy,
-                                                   const W *__restrict__ wz, S a, int at)
+                                                   const W *__restrict__ wz, const InvRows<R> &M,
+                                                   int at)
 {
-    using R = typename std::remove_reference<decltype(*a.a)>::type;
     const int m = nx * ny * nz;
     for (int r = threadIdx.x; r < m; r += blockDim.x) {
+        R *row = M.own(at + r);
+        if (!row) continue;
         const int i = r % nx, j = (r / nx) % ny, k = r / (nx * ny);
         const long long c = (long long)k * Q + (long long)j * P + i;
         const W ww = wx[c], we = wx[c + 1], ws = wy[c], wn = wy[c + P], wd = wz[c],
                 wu = wz[c + Q];
-        R *row = a.row(at + r);
         row[0] = (R)(((ww + we) + (ws + wn)) + (wd + wu));
         if (i < nx - 1) row[1] = (R)-we;
         if (j < ny - 1) row[nx] = (R)-wn;
@@ -1873,83 +1903,124 @@ __device__ __forceinline__ void assemble_box_block(int nx, int ny, int nz, int P
     }
 }
 
-template <class R, class S>
-__device__ __forceinline__ void gauss_jordan_cta(S a, int n, bool singular, double *inv64,
-                                                 float *inv32, R *col);
-
-// The coarsest level's inverse in precision R (double: A^{-1} to inv64 and
-// its rounding to inv32; float, when no FP64 inverse is wanted: inv32 only).
-// a: the matrix storage (SymStore of R, n = the box's cells); col: 2n of R
-// (shared memory).
-template <class R, class S, class W>
-__device__ __forceinline__ void bottom_inverse_cta(int nx, int ny, int nz, int P, long long Q,
-                                                   const W *__restrict__ wx,
-                                                   const W *__restrict__ wy,
-                                                   const W *__restrict__ wz, bool singular,
-                                                   S a, double *inv64, float *inv32, R *col)
+// The matrix storage of a cluster's inverse: two columns and the pivot row
+// first (3 n of R), then the rows if they fit in smem_bytes, else scratch.
+template <class R>
+__device__ __forceinline__ InvRows<R> inv_rows(const cg::cluster_group &cl, int n, R *smem,
+                                               int smem_bytes, R *scratch)
 {
-    for (long long e = threadIdx.x; e < a.size(); e += blockDim.x) a.a[e] = R(0);
+    InvRows<R> M;
+    M.n = n;
+    M.rank = (int)cl.block_rank();
+    M.ncta = (int)cl.num_blocks();
+    M.packed = (3LL * n + inv_rows_elems(n, M.ncta)) * (long long)sizeof(R) <= smem_bytes;
+    M.a = M.packed ? smem + 3 * n : scratch;
+    for (int m = threadIdx.x >> 5; m < M.count(); m += kInvThreads / 32) {
+        R *r = M.row(m);
+        for (int j = threadIdx.x & 31; j < n - M.rank - M.ncta * m; j += 32) r[j] = R(0);
+    }
     __syncthreads();
-    assemble_box_block(nx, ny, nz, P, Q, wx, wy, wz, a, 0);
-    __syncthreads();
-    gauss_jordan_cta(a, a.n, singular, inv64, inv32, col);
+    return M;
 }
 
-// In-place Gauss-Jordan inverse of M (symmetric positive definite; with
-// `singular` first shifted by c 1 1^T as described above), written as
-// A^{-1} = -M^{-1} to inv64 and/or inv32 (either may be NULL).  Pivots are
-// taken in order, without exchanges (M is diagonally dominant or positive
-// definite), and only the upper triangle is kept: after pivots 0..p an entry
-// with exactly one index <= p is the negative of its mirror and every other
-// entry equals its mirror, so the lower triangle follows from the upper one
-// and each pivot costs n^2/2 updates instead of n^2 (the FP64 pipe of the
-// single SM that inverts a box is the limit once the matrix sits in shared
-// memory).  a: SymStore of R; col: 2n of R.
-template <class R, class S>
-__device__ __forceinline__ void gauss_jordan_cta(S a, int n, bool singular, double *inv64,
-                                                 float *inv32, R *col)
+// Invert the assembled rows; A^{-1} to inv64 and/or inv32 (either may be NULL).
+// smem: the columns and the pivot row; ips: shared, [2].
+template <class R>
+__device__ __forceinline__ void gauss_jordan_cluster(const cg::cluster_group &cl,
+                                                     const InvRows<R> &M, bool singular,
+                                                     double *inv64, float *inv32, R *smem, R *ips)
 {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-    R *rowv = col + n;
+    const int n = M.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nw = kInvThreads / 32, rows = M.count();
+    R *const rowv = smem + 2 * n;
+    auto everywhere = [&](R *p, R v) {
+        for (int r = 0; r < M.ncta; ++r) *cl.map_shared_rank(p, r) = v;
+    };
+    cl.sync();   // every CTA's shared memory is in use
     if (singular) {
+        for (int m = tid; m < rows; m += kInvThreads) everywhere(smem + M.rank + M.ncta * m, M.row(m)[0]);
+        cl.sync();
         if (tid == 0) {
             R tr = R(0);
-            for (int r = 0; r < n; ++r) tr += a(r, r);
-            col[0] = tr / ((R)n * (R)n);
+            for (int r = 0; r < n; ++r) tr += smem[r];
+            ips[0] = tr / ((R)n * (R)n);
         }
         __syncthreads();
-        const R shift = col[0];
-        __syncthreads();
-        for (long long e = tid; e < a.size(); e += nt) a.a[e] += shift;
-        __syncthreads();
+        const R shift = ips[0];
+        for (int m = warp; m < rows; m += nw) {
+            R *r = M.row(m);
+            for (int j = lane; j < n - M.rank - M.ncta * m; j += 32) r[j] += shift;
+        }
+        cl.sync();
     }
+    if (M.rank == 0) {   // the first pivot's column is row 0
+        const R *r = M.row(0);
+        for (int j = tid; j < n; j += kInvThreads) everywhere(smem + j, r[j]);
+        if (tid == 0) everywhere(ips, R(1) / r[0]);
+    }
+    cl.sync();
     for (int p = 0; p < n; ++p) {
-        // column p (the entries below the diagonal mirror those of row p)
-        for (int i = tid; i < n; i += nt) col[i] = i <= p ? a(i, p) : a(p, i);
+        // column p: (i, p) for i <= p, (p, i) below the diagonal; its new row
+        // p: a_pj / a_pp (a_pj for j < p is minus its stored mirror)
+        const R *const col = smem + (p & 1) * n;
+        R *const next = smem + ((p + 1) & 1) * n;
+        const R ip = ips[p & 1];
+        for (int j = tid; j < n; j += kInvThreads)
+            rowv[j] = j == p ? ip : (j > p ? col[j] : -col[j]) * ip;
         __syncthreads();
-        const R ip = R(1) / col[p];
-        // new row p: a_pj / a_pp (a_pj for j < p is minus its stored mirror)
-        for (int j = tid; j < n; j += nt)
-            rowv[j] = j == p ? ip : (j > p ? a(p, j) : -a(j, p)) * ip;
-        __syncthreads();
-        for (int i = warp; i < n; i += nw) {
+        for (int m = warp; m < rows; m += nw) {
+            const int i = M.rank + M.ncta * m;
             const R ci = col[i];
-            R *ar = a.row(i);
+            R *ar = M.row(m);
             for (int j = i + lane; j < n; j += 32) {
-                if (i == p) ar[j - i] = rowv[j];             // row p (j >= p; j = p: 1 / a_pp)
-                else if (j == p) ar[j - i] = -ci * ip;       // column p above the diagonal
-                else ar[j - i] -= ci * rowv[j];
+                R v;
+                if (i == p) v = rowv[j];              // row p (j >= p; j = p: 1 / a_pp)
+                else if (j == p) v = -ci * ip;        // column p above the diagonal
+                else v = fmadd(-ci, rowv[j], ar[j - i]);
+                ar[j - i] = v;
+                if (j == p + 1) {                     // column p + 1, down to its diagonal
+                    everywhere(next + i, v);
+                    if (i == p + 1) everywhere(ips + ((p + 1) & 1), R(1) / v);
+                } else if (i == p + 1) {              // and, mirrored, from row p + 1
+                    everywhere(next + j, v);
+                }
             }
         }
-        __syncthreads();
+        cl.sync();
     }
-    for (long long e = tid; e < (long long)n * n; e += nt) {
-        const int i = (int)(e / n), j = (int)(e % n);
-        const double v = -(double)(i <= j ? a(i, j) : a(j, i));
-        if (inv64) inv64[e] = v;
-        if (inv32) inv32[e] = (float)v;
+    for (int m = warp; m < rows; m += nw) {
+        const int i = M.rank + M.ncta * m;
+        const R *ar = M.row(m);
+        for (int j = i + lane; j < n; j += 32) {
+            const double v = -(double)ar[j - i];
+            const long long e = (long long)i * n + j, t = (long long)j * n + i;
+            if (inv64) {
+                inv64[e] = v;
+                inv64[t] = v;
+            }
+            if (inv32) {
+                inv32[e] = (float)v;
+                inv32[t] = (float)v;
+            }
+        }
     }
+}
+
+// The coarsest level's inverse of one box in precision R (double: A^{-1} to
+// inv64 and its rounding to inv32; float, when no FP64 inverse is wanted: inv32
+// only), by the calling cluster.
+template <class R, class W>
+__device__ __forceinline__ void bottom_inverse_cluster(const cg::cluster_group &cl, int nx, int ny,
+                                                       int nz, int P, long long Q,
+                                                       const W *__restrict__ wx,
+                                                       const W *__restrict__ wy,
+                                                       const W *__restrict__ wz, bool singular,
+                                                       R *smem, int smem_bytes, R *scratch,
+                                                       double *inv64, float *inv32, R *ips)
+{
+    const InvRows<R> M = inv_rows<R>(cl, nx * ny * nz, smem, smem_bytes, scratch);
+    assemble_box_block(nx, ny, nz, P, Q, wx, wy, wz, M, 0);
+    gauss_jordan_cluster<R>(cl, M, singular, inv64, inv32, smem, ips);
 }
 
 // ---- one box (single-stage entry points): grid over positions
@@ -2002,24 +2073,16 @@ __global__ void k_round_f32(int nx, int ny, int nz, int P, long long Q, const do
     round_at(nx, ny, nz, P, Q, wx, wy, wz, invD, wx32, wy32, wz32, invD32, i, j, k);
 }
 
-__global__ void __launch_bounds__(1024) k_bottom_inverse(int nx, int ny, int nz, int P, long long Q,
-                                                         const double *__restrict__ wx,
-                                                         const double *__restrict__ wy,
-                                                         const double *__restrict__ wz,
-                                                         int singular, double *__restrict__ a,
-                                                         double *__restrict__ inv64,
-                                                         float *__restrict__ inv32, int packed)
+__global__ void __launch_bounds__(kInvThreads) k_bottom_inverse(
+    int nx, int ny, int nz, int P, long long Q, const double *__restrict__ wx,
+    const double *__restrict__ wy, const double *__restrict__ wz, int singular,
+    double *__restrict__ a, double *__restrict__ inv64, float *__restrict__ inv32, int smem_bytes)
 {
-    __shared__ double col[2 * MG_BOTTOM_CELLS];
-    extern __shared__ __align__(16) unsigned char bottom_packed[];
-    const int n = nx * ny * nz;
-    if (packed)
-        bottom_inverse_cta<double>(nx, ny, nz, P, Q, wx, wy, wz, singular != 0,
-                                   SymStore<double, true>{reinterpret_cast<double *>(bottom_packed), n},
-                                   inv64, inv32, col);
-    else
-        bottom_inverse_cta<double>(nx, ny, nz, P, Q, wx, wy, wz, singular != 0,
-                                   SymStore<double, false>{a, n}, inv64, inv32, col);
+    extern __shared__ __align__(16) unsigned char inv_smem[];
+    __shared__ double ips[2];
+    bottom_inverse_cluster<double>(cg::this_cluster(), nx, ny, nz, P, Q, wx, wy, wz, singular != 0,
+                                   reinterpret_cast<double *>(inv_smem), smem_bytes, a, inv64,
+                                   inv32, ips);
 }
 
 // ---- every box of a level in one launch (the solver's set-up)
@@ -2091,53 +2154,29 @@ __global__ void __launch_bounds__(kThreads) k_setup(SetupSet S, int t0)
     setup_step<STEP>(B, p);
 }
 
-// One CTA per box: the coarsest level's dense inverse, in FP64 when an FP64
-// inverse is wanted, else (mixed precision, whose FP64 levels never solve)
-// in FP32 straight away; a matrix whose packed upper triangle fits in the
-// launch's dynamic shared memory (packed_bytes, at most kPackedBottomBytes)
-// is inverted there, a larger one in the box's global scratch.
-__global__ void __launch_bounds__(1024) k_setup_bottom(SetupSet S, int packed_bytes)
+// One cluster per box: the coarsest level's dense inverse, in FP64 when an FP64
+// inverse is wanted, else (mixed precision, whose FP64 levels never solve) in
+// FP32 straight away.
+__global__ void __launch_bounds__(kInvThreads) k_setup_bottom(SetupSet S, int smem_bytes)
 {
-    __shared__ double col[2 * MG_BOTTOM_CELLS];
-    extern __shared__ __align__(16) unsigned char bottom_packed[];
-    const SetupBox &B = S.boxes[blockIdx.x];
+    extern __shared__ __align__(16) unsigned char inv_smem[];
+    __shared__ double ips[2];
+    const cg::cluster_group cl = cg::this_cluster();
+    const SetupBox &B = S.boxes[blockIdx.x / cl.num_blocks()];
     const bool singular = (B.bc & 63) == 63;
-    const int n = B.nx * B.ny * B.nz;
-    const long long tri = (long long)n * (n + 1) / 2;
-    if (B.w32src) {
+    double *const sd = reinterpret_cast<double *>(inv_smem);
+    float *const sf = reinterpret_cast<float *>(inv_smem), *const wf = reinterpret_cast<float *>(B.work);
+    float *const ipf = reinterpret_cast<float *>(ips);
+    if (B.w32src)
         // coarser FP32 levels averaged in FP32: assembled from their weights
-        float *colf = reinterpret_cast<float *>(col);
-        if (tri * (long long)sizeof(float) <= packed_bytes)
-            bottom_inverse_cta<float>(
-                B.nx, B.ny, B.nz, B.P, B.Q, B.wx32, B.wy32, B.wz32, singular,
-                SymStore<float, true>{reinterpret_cast<float *>(bottom_packed), n}, nullptr,
-                B.inv32, colf);
-        else
-            bottom_inverse_cta<float>(B.nx, B.ny, B.nz, B.P, B.Q, B.wx32, B.wy32, B.wz32,
-                                      singular,
-                                      SymStore<float, false>{reinterpret_cast<float *>(B.work), n},
-                                      nullptr, B.inv32, colf);
-    } else if (B.inv64) {
-        if (tri * (long long)sizeof(double) <= packed_bytes)
-            bottom_inverse_cta<double>(
-                B.nx, B.ny, B.nz, B.P, B.Q, B.wx, B.wy, B.wz, singular,
-                SymStore<double, true>{reinterpret_cast<double *>(bottom_packed), n}, B.inv64,
-                B.inv32, col);
-        else
-            bottom_inverse_cta<double>(B.nx, B.ny, B.nz, B.P, B.Q, B.wx, B.wy, B.wz, singular,
-                                       SymStore<double, false>{B.work, n}, B.inv64, B.inv32, col);
-    } else {
-        float *colf = reinterpret_cast<float *>(col);
-        if (tri * (long long)sizeof(float) <= packed_bytes)
-            bottom_inverse_cta<float>(
-                B.nx, B.ny, B.nz, B.P, B.Q, B.wx, B.wy, B.wz, singular,
-                SymStore<float, true>{reinterpret_cast<float *>(bottom_packed), n}, nullptr,
-                B.inv32, colf);
-        else
-            bottom_inverse_cta<float>(B.nx, B.ny, B.nz, B.P, B.Q, B.wx, B.wy, B.wz, singular,
-                                      SymStore<float, false>{reinterpret_cast<float *>(B.work), n},
-                                      nullptr, B.inv32, colf);
-    }
+        bottom_inverse_cluster<float>(cl, B.nx, B.ny, B.nz, B.P, B.Q, B.wx32, B.wy32, B.wz32,
+                                      singular, sf, smem_bytes, wf, nullptr, B.inv32, ipf);
+    else if (B.inv64)
+        bottom_inverse_cluster<double>(cl, B.nx, B.ny, B.nz, B.P, B.Q, B.wx, B.wy, B.wz, singular,
+                                       sd, smem_bytes, B.work, B.inv64, B.inv32, ips);
+    else
+        bottom_inverse_cluster<float>(cl, B.nx, B.ny, B.nz, B.P, B.Q, B.wx, B.wy, B.wz, singular,
+                                      sf, smem_bytes, wf, nullptr, B.inv32, ipf);
 }
 
 // ----------------------------------------------------- projection steps ----
@@ -2627,20 +2666,21 @@ __global__ void __launch_bounds__(kThreads) k_guard_fill(BoxSet<T> S, T v)
     }
 }
 
-// Dense inverse of the union of the boxes' coarsest levels (one CTA): each
+// Dense inverse of the union of the boxes' coarsest levels (one cluster): each
 // box's block as for a single box, plus -w between a box's cell and the cell
 // of the neighbouring box (or, on a periodic axis, of the box itself) across
 // every exchanged face (from the coarsest level's exchange records: guard
 // cell of dst <-> cell of src), then Gauss-Jordan (with the constant shift
 // when A is singular).  S: the coarsest level of every box, in union order.
-__global__ void __launch_bounds__(1024) k_union_inverse(SetupSet S, UnionBottom U, double *a,
-                                                        double *inv64, float *inv32)
+__global__ void __launch_bounds__(kInvThreads) k_union_inverse(SetupSet S, UnionBottom U, double *a,
+                                                               double *inv64, float *inv32,
+                                                               int smem_bytes)
 {
-    __shared__ double col[2 * MG_BOTTOM_CELLS];
-    const int n = U.n;
-    const SymStore<double, false> M{a, n};
-    for (long long e = threadIdx.x; e < (long long)n * n; e += blockDim.x) a[e] = 0.0;
-    __syncthreads();
+    extern __shared__ __align__(16) unsigned char inv_smem[];
+    __shared__ double ips[2];
+    const cg::cluster_group cl = cg::this_cluster();
+    double *const sd = reinterpret_cast<double *>(inv_smem);
+    const InvRows<double> M = inv_rows<double>(cl, U.n, sd, smem_bytes, a);
     for (int b = 0; b < U.nbox; ++b) {
         const SetupBox &B = S.boxes[b];
         assemble_box_block(B.nx, B.ny, B.nz, B.P, B.Q, B.wx, B.wy, B.wz, M, U.off[b]);
@@ -2668,14 +2708,17 @@ __global__ void __launch_bounds__(1024) k_union_inverse(SetupSet S, UnionBottom 
             else if (gk < 0) w = D.wz[c];
             else w = D.wz[c + D.Q];
             const int row = U.off[R.dst] + (ck * D.ny + cj) * D.nx + ci;
-            const int cl = U.off[R.src] + (sk * F.ny + sj) * F.nx + si;
+            const int col = U.off[R.src] + (sk * F.ny + sj) * F.nx + si;
             // added, not set: across a periodic axis of 2 cells the same two
             // cells are also neighbours through the inner face
-            a[(long long)row * n + cl] -= w;
+            if (col >= row) {
+                double *r = M.own(row);
+                if (r) r[col - row] -= w;
+            }
         }
         __syncthreads();
     }
-    gauss_jordan_cta(M, n, U.singular != 0, inv64, inv32, col);
+    gauss_jordan_cluster<double>(cl, M, U.singular != 0, inv64, inv32, sd, ips);
 }
 
 // Coarsest solve of a coupled level: phi = Ainv f over the union, rows in
@@ -3437,35 +3480,50 @@ cudaError_t launch_round_f32(int nx, int ny, int nz, const double *wx, const dou
     return counted(cudaGetLastError());
 }
 
-int packed_bottom_bytes(int n, bool fp64)
+// CTAs of the cluster that inverts an n x n matrix (nbox of them at once), and
+// the shared memory of each: short matrices are a chain of barriers, which one
+// CTA passes fastest.
+static int inv_ctas(int n, int nbox)
 {
-    const long long b = (long long)n * (n + 1) / 2 * (fp64 ? 8 : 4);
-    return b <= kPackedBottomBytes ? (int)b : 0;
+    int c = n >= 128 ? 16 : n >= 48 ? 8 : 1;
+    while (c > 1 && (long long)c * nbox > 304) c /= 2;   // (two waves of CTAs)
+    return c;
+}
+static int inv_bytes(int n, int ctas, bool fp64)
+{
+    const long long e = fp64 ? 8 : 4, rows = (3LL * n + inv_rows_elems(n, ctas)) * e;
+    return (int)(rows <= kTailSmem ? rows : 3LL * n * e);
 }
 
-// the dense inverses' packed matrices: dynamic shared memory beyond 48 KB
-static void bottom_smem_attributes()
+template <class K, class... Args>
+static cudaError_t inv_launch(K kernel, int clusters, int ctas, int smem, cudaStream_t st, Args... args)
 {
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_bottom_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kPackedBottomBytes);
-        cudaFuncSetAttribute(k_setup_bottom, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kPackedBottomBytes);
-        cudaGetLastError();
-    });
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmem);
+    if (e == cudaSuccess && ctas > 8)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(clusters * ctas);
+    cfg.blockDim = dim3(kInvThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ctas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return counted(cudaLaunchKernelEx(&cfg, kernel, args...));
 }
 
 cudaError_t launch_bottom_inverse(int nx, int ny, int nz, const double *wx, const double *wy,
                                   const double *wz, int singular, double *work, double *inv64,
                                   float *inv32, cudaStream_t st)
 {
-    const int packed = packed_bottom_bytes(nx * ny * nz, true);
-    bottom_smem_attributes();
-    k_bottom_inverse<<<1, 1024, packed, st>>>(nx, ny, nz, (int)pitch_row(nx), pitch_plane(nx, ny),
-                                              wx, wy, wz, singular, work, inv64, inv32,
-                                              packed > 0 ? 1 : 0);
-    return counted(cudaGetLastError());
+    const int n = nx * ny * nz, c = inv_ctas(n, 1), smem = inv_bytes(n, c, true);
+    return inv_launch(k_bottom_inverse, 1, c, smem, st, nx, ny, nz, (int)pitch_row(nx),
+                      (long long)pitch_plane(nx, ny), wx, wy, wz, singular, work, inv64, inv32, smem);
 }
 
 cudaError_t launch_setup_tiles(const SetupSet &S, int step, int t0, int t1, cudaStream_t st)
@@ -3493,12 +3551,11 @@ cudaError_t launch_setup(const SetupSet &S, int step, cudaStream_t st)
     return launch_setup_tiles(S, step, 0, S.ntiles[setup_kind(step)], st);
 }
 
-cudaError_t launch_setup_bottom(const SetupSet &S, int packed_bytes, cudaStream_t st)
+cudaError_t launch_setup_bottom(const SetupSet &S, int max_cells, bool fp64, cudaStream_t st)
 {
     if (S.nbox == 0) return cudaSuccess;
-    bottom_smem_attributes();
-    k_setup_bottom<<<S.nbox, 1024, packed_bytes, st>>>(S, packed_bytes);
-    return counted(cudaGetLastError());
+    const int c = inv_ctas(max_cells, S.nbox), smem = inv_bytes(max_cells, c, fp64);
+    return inv_launch(k_setup_bottom, S.nbox, c, smem, st, S, smem);
 }
 
 cudaError_t launch_project_rhs(int nx, int ny, int nz, double h, const double *u, const double *v,
@@ -3666,8 +3723,8 @@ cudaError_t launch_guard_fill(const BoxSet<T> &S, T v, cudaStream_t st)
 cudaError_t launch_union_inverse(const SetupSet &S, const UnionBottom &U, double *work,
                                  double *inv64, float *inv32, cudaStream_t st)
 {
-    k_union_inverse<<<1, 1024, 0, st>>>(S, U, work, inv64, inv32);
-    return counted(cudaGetLastError());
+    const int c = inv_ctas(U.n, 1), smem = inv_bytes(U.n, c, true);
+    return inv_launch(k_union_inverse, 1, c, smem, st, S, U, work, inv64, inv32, smem);
 }
 
 template <class T>

@@ -243,13 +243,9 @@ cudaError_t launch_setup(const SetupSet &S, int step, cudaStream_t st);
 // Tiles [t0, t1) of one step (tiles are numbered plane by plane, so a range
 // of whole planes of a one-box set is a range of tiles).
 cudaError_t launch_setup_tiles(const SetupSet &S, int step, int t0, int t1, cudaStream_t st);
-// The coarsest level's dense inverse, one CTA per box.
-// packed_bytes: dynamic shared memory for the packed upper triangles (the
-// largest packed_bottom_bytes over the boxes; 0: every matrix in scratch)
-cudaError_t launch_setup_bottom(const SetupSet &S, int packed_bytes, cudaStream_t st);
-// Bytes of the packed upper triangle of an n-cell coarsest matrix if it is
-// inverted in shared memory, else 0.
-int packed_bottom_bytes(int n, bool fp64);
+// The coarsest level's dense inverse, one cluster per box: max_cells of the
+// largest, fp64 whether FP64 inverses are wanted.
+cudaError_t launch_setup_bottom(const SetupSet &S, int max_cells, bool fp64, cudaStream_t st);
 
 // Projection steps (natural layouts): f = div(u, v, w) - S (S nullable), and
 // u, v, w -= beta_face grad(phi) using the level-0 weights.

@@ -1150,10 +1150,6 @@ int solver_create(Solver **out, int nbox, const int (*n)[3], const double *dx, i
     {
         std::vector<SetupBox> bot;
         for (int b = 0; b < nsetup; ++b) bot.push_back(setup_box(b, s->nlev[b] - 1));
-        s->bottom_packed = 0;
-        for (const SetupBox &B : bot)
-            s->bottom_packed = std::max(s->bottom_packed,
-                                        packed_bottom_bytes(B.nx * B.ny * B.nz, B.inv64 != nullptr));
         psu.push_back(plan_set(blob, &s->setup_bottom, bot));
     }
     // ghost exchange records of every level and the union numbering of the
@@ -1446,13 +1442,13 @@ int solver_set_beta(Solver *s, const double *beta, cudaStream_t st)
             CK(launch_setup(s->setup_coarsen[l], 1, st));
     }
     // the dense coarsest inverses need the coarsest weights only: forked to
-    // the side stream (one CTA per box, on as many SMs), they overlap the
+    // the side stream (one cluster per box), they overlap the
     // diagonal and FP32 steps of the finer levels on the others (with
     // coarse32 those came first: the coarsest FP32 weights end that chain)
     if (!s->xmode) {
         CK(cudaEventRecord(s->ev_fork, st));
         CK(cudaStreamWaitEvent(s->side, s->ev_fork, 0));
-        if (!s->cg_bottom) CK(launch_setup_bottom(s->setup_bottom, s->bottom_packed, s->side));
+        if (!s->cg_bottom) CK(launch_setup_bottom(s->setup_bottom, s->max_bottom, !s->has32, s->side));
         CK(cudaEventRecord(s->ev_join, s->side));
     }
     for (int l = 0; l < s->maxlev && !c32; ++l) {
@@ -1482,7 +1478,7 @@ int solver_setup_from_weights(Solver *s, cudaStream_t st)
     CK(cudaEventRecord(s->ev_setup0, st));
     const long long k0 = launch_counter();
     for (size_t l = 0; l < s->setup_coarsen.size(); ++l) CK(launch_setup(s->setup_coarsen[l], 1, st));
-    if (!s->cg_bottom) CK(launch_setup_bottom(s->setup_bottom, s->bottom_packed, st));
+    if (!s->cg_bottom) CK(launch_setup_bottom(s->setup_bottom, s->max_bottom, !s->has32, st));
     for (int l = 0; l < s->maxlev; ++l) CK(launch_setup(s->setup_lv[l], 2, st));
     CK(cudaEventRecord(s->ev_setup1, st));
     s->kernels += launch_counter() - k0;

@@ -169,7 +169,6 @@ struct Solver {
     std::vector<SetupSet> setup_lv;       // [level] every box that has the level
     std::vector<SetupSet> setup_coarsen;  // [level] boxes that have level + 1
     SetupSet setup_bottom{};              // coarsest level of every box
-    int bottom_packed = 0;                // dynamic shared memory of k_setup_bottom (packed matrices)
 
     int *derr = nullptr;                  // device error word (bounded waits that gave up)
     unsigned *gbar = nullptr;             // device grid-barrier word of the persistent launches

@@ -68,3 +68,37 @@ def test_cluster_sizes_of_batches(cuda_device, nbox):
         s.close()
     assert out[0][1] == out[1][1]
     assert np.linalg.norm(out[1][0] - out[0][0]) <= 1e-12 * np.linalg.norm(out[0][0])
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1), (3, 5, 3), (4, 4, 3), (7, 3, 6), (8, 8, 2), (5, 9, 17),
+                                   (9, 10, 11), (8, 8, 16)])
+@pytest.mark.parametrize("singular", [False, True])
+def test_cluster_inverse(cuda_device, shape, singular):
+    # one, eight and sixteen CTAs, rows in shared memory and (1024) in scratch:
+    # A Ainv against the identity, less the constant part when A is singular.
+    # Backward error of an elimination without exchanges on a diagonally
+    # dominant matrix: a few n eps |A| |Ainv|.
+    from paper_1008_2801_gb300 import ops as K
+
+    rng = np.random.default_rng(71)
+    beta = torch.from_numpy(rng.uniform(0.5, 2.0, shape)).to(cuda_device)
+    if singular and beta.numel() == 1:
+        pytest.skip("A is 0")
+    w = K.face_weights(beta, 1.0, bc=63 if singular else 0)
+    inv = K.bottom_inverse(w, shape, singular).cpu().numpy()
+    wx, wy, wz = (K.get(t, shape, k).cpu().numpy() for t, k in zip(w, "xyz"))
+    n = inv.shape[0]
+    idx = np.arange(n).reshape(shape)
+    A = np.zeros((n, n))
+    np.fill_diagonal(A, -(wx[:, :, :-1] + wx[:, :, 1:] + wy[:, :-1] + wy[:, 1:] + wz[:-1]
+                          + wz[1:]).ravel())
+    for a, b, v in ((idx[:, :, :-1], idx[:, :, 1:], wx[:, :, 1:-1]),
+                    (idx[:, :-1], idx[:, 1:], wy[:, 1:-1]), (idx[:-1], idx[1:], wz[1:-1])):
+        A[a.ravel(), b.ravel()] = v.ravel()
+        A[b.ravel(), a.ravel()] = v.ravel()
+    assert np.array_equal(inv, inv.T)
+    eye = np.eye(n) - (1.0 / n if singular else 0.0)
+    if singular:   # on zero-mean right-hand sides
+        inv = inv @ eye
+    bar = 8 * n * 2.0 ** -53 * np.linalg.norm(A, 1) * np.linalg.norm(inv, 1)
+    assert np.abs(A @ inv - eye).max() <= bar
