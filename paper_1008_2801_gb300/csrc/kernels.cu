@@ -192,6 +192,18 @@ __device__ __forceinline__ double rcp64(double d)
     return fma(fma(e, e, e), y, y);
 }
 
+// Tile of this CTA in a launch that runs its tiles backwards.  Consecutive
+// kernels of a level alternate direction (red passes, restrictions and the
+// norm pass forwards, black passes and prolongations backwards), so that each
+// starts on what the one before left in L2 (126 MB; a batch of 64 boxes of 64^3
+// takes 29.6 ms against 30.6 with every kernel forwards, a 256^3 solve
+// 16.56 against 16.8, 512^3, where L2 holds a twentieth of a pass, 130.0
+// against 130.2).  No kernel reads what another tile of its own launch wrote.
+__device__ __forceinline__ int tile_dir(bool back)
+{
+    return back ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
+}
+
 // ---------------------------------------------- single-colour GS pass ----
 
 // The value of a boundary cell into its copies in neighbouring guard cells.
@@ -228,7 +240,7 @@ __global__ void __launch_bounds__(kThreads) k_rbgs_pass(BoxSet<T> S, const int *
                                                         int color)
 {
     pdl_wait();
-    const int t = blockIdx.x;
+    const int t = tile_dir(color != 0);
     const int *ts = S.tstart[TK_PAIR];
     const int b = find_box(ts, S.nbox, t);
     const Box<T> &B = S.boxes[b];
@@ -309,7 +321,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_rbgs_pass_oop(BoxSet<T> S,
                                                                int color, int from2)
 {
     pdl_wait();
-    const int t = blockIdx.x;
+    const int t = tile_dir(color != 0);
     const int *ts = S.tstart[TK_PAIR];
     const int b = find_box(ts, S.nbox, t);
     const Box<T> &B = S.boxes[b];
@@ -721,7 +733,7 @@ template <class T, bool FC>
 __global__ void __launch_bounds__(kThreads) k_prolong(BoxSet<T> S, const int *__restrict__ active)
 {
     pdl_wait();
-    prolong_tile<T, FC>(S, active, blockIdx.x);
+    prolong_tile<T, FC>(S, active, tile_dir(true));
 }
 
 // -------------------------------------------------------- residual field ----
@@ -2801,7 +2813,7 @@ __global__ void __launch_bounds__(kThreads) k_rbgs_pass_multi(BoxSet<T> S,
     const Box<T> &B0 = S.boxes[0];
     const int P = B0.P;
     const long long Q = B0.Q;
-    const TilePos p = tile_pos(TK_PAIR, B0.nx, B0.ny, B0.nz, blockIdx.x);
+    const TilePos p = tile_pos(TK_PAIR, B0.nx, B0.ny, B0.nz, tile_dir(color != 0));
     const int j = p.y, k = p.z;
     const int i = 2 * p.x + ((j + k + color + B0.par) & 1);
     if (j >= B0.ny || i >= B0.nx) return;
@@ -2834,7 +2846,7 @@ __global__ void __launch_bounds__(kThreads) k_rbgs_pass_oop_multi(BoxSet<T> S,
     const Box<T> &B0 = S.boxes[0];
     const int P = B0.P;
     const long long Q = B0.Q;
-    const TilePos p = tile_pos(TK_PAIR, B0.nx, B0.ny, B0.nz, blockIdx.x);
+    const TilePos p = tile_pos(TK_PAIR, B0.nx, B0.ny, B0.nz, tile_dir(color != 0));
     const int j = p.y, k = p.z, x0 = 2 * p.x;
     if (j >= B0.ny || x0 >= B0.nx) return;
     typedef typename Vec2<T>::type V2;
