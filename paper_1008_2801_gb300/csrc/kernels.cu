@@ -3138,7 +3138,7 @@ __global__ void __launch_bounds__(kThreads) k_cg_bottom(BoxSet<T> S, const int *
         }
     };
     auto put = [&](double *dst, double v) {
-        const double bs = block_sum(v);
+        const double bs = block_sum_ordered(v);
         if (threadIdx.x == 0 && threadIdx.y == 0) dst[blockIdx.x] = bs;
     };
     // x = 0, r = -f, p = D^-1 r, partial <r, D^-1 r>
