@@ -3197,6 +3197,108 @@ __global__ void __launch_bounds__(kThreads) k_cg_bottom(BoxSet<T> S, const int *
     }
 }
 
+// The same iteration, the same bits, by one cluster when the level has at most
+// 16 x 2 cell tiles: a thread holds its cell's x, r, weights and 1/D in
+// registers through the solve, only p is in memory, a tile's partial sums go
+// into every CTA through distributed shared memory, and the three barriers of
+// an iteration are the cluster's.  What bounds it: the barriers, the dependent
+// FP64 sums (8 + 5 + 5 of ~100 cycles), p's round trip through L2 and the
+// FP64 pipes of 16 SMs, which set the line: FP64 solves of 36 x 52 x 44 cells
+// (11 tiles) 7.1 -> 4.0 ms, 13 x 9 x 9 (13) 0.74 -> 0.46, 104 x 120 x 152 (26)
+// 13.1 -> 10.6; with four tiles a CTA 168 x 176 x 240 (60 tiles) took 26.8 ms
+// against 24.6 and 64 x 17 x 15 (64) 2.2 against 1.8.
+constexpr int kCgCtas = 16, kCgGroups = 2;
+
+template <class T>
+__global__ void __launch_bounds__(kThreads *kCgGroups)
+    k_cg_bottom_cluster(BoxSet<T> S, const int *__restrict__ active, T *p, double tol, int maxit)
+{
+    const cg::cluster_group cl = cg::this_cluster();
+    const Box<T> &B = S.boxes[0];
+    if (active && !active[B.box]) return;
+    __shared__ double wpart[kThreads / 32 * kCgGroups], part[2][kCgCtas * kCgGroups], tot;
+    const int nt = S.ntiles[TK_CELL], CL = (int)cl.num_blocks();
+    const int t = (int)threadIdx.z * CL + (int)cl.block_rank();
+    const int warp = (int)threadIdx.z * kTY + (int)threadIdx.y, lane = threadIdx.x;
+    const TilePos tp = tile_pos(TK_CELL, B.nx, B.ny, B.nz, t);
+    const bool on = t < nt && tp.x < B.nx && tp.y < B.ny;
+    const int P = B.P;
+    const long long Q = B.Q;
+    const long long c = on ? (long long)tp.z * Q + (long long)tp.y * P + tp.x : 0;
+    // the sum over all cells of v, in the order of the cooperative launch with
+    // one tile a CTA (w: which of two buffers, used in turn)
+    auto total = [&](double v, int w) {
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) wpart[warp] = v;
+        __syncthreads();
+        if (threadIdx.y == 0 && t < nt) {
+            double s = 0.0;
+            for (int i = 0; i < kThreads / 32; ++i) s += wpart[warp + i];
+            if (lane < CL) cl.map_shared_rank(&part[w][0], lane)[t] = s;
+        }
+        cl.sync();
+        if (warp == 0) {
+            double s = 0.0;
+            for (int i = lane; i < nt; i += 32) s += part[w][i];
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+            if (lane == 0) tot = s;
+        }
+        __syncthreads();
+        return tot;
+    };
+    T wxa = 0, wxb = 0, wya = 0, wyb = 0, wza = 0, wzb = 0, D = 0, id = 0, x = 0, r = 0, pc = 0;
+    if (on) {
+        const long long cf = fidx(B, tp.x, tp.y, tp.z);
+        wxa = B.wx[c];
+        wxb = B.wx[c + 1];
+        wya = B.wy[c];
+        wyb = B.wy[c + P];
+        wza = B.wz[c];
+        wzb = B.wz[c + Q];
+        D = B.D ? B.D[cf] : ((wxa + wxb) + (wya + wyb)) + (wza + wzb);
+        id = B.invD[cf];
+        r = -B.f[cf];
+        pc = r * id;
+        p[c] = pc;
+    }
+    cl.sync();   // every CTA runs before its shared memory is written
+    double rz = total((double)r * (double)pc, 1);
+    const double stop = tol * tol * rz;
+    double best = rz;
+    int since = 0;
+    for (int it = 0; it < maxit && rz > 0.0; ++it) {
+        T q = 0;
+        if (on) {
+            q = D * pc;
+            q = fmadd(-wxa, __ldcg(p + c - 1), q);
+            q = fmadd(-wxb, __ldcg(p + c + 1), q);
+            q = fmadd(-wya, __ldcg(p + c - P), q);
+            q = fmadd(-wyb, __ldcg(p + c + P), q);
+            q = fmadd(-wza, __ldcg(p + c - Q), q);
+            q = fmadd(-wzb, __ldcg(p + c + Q), q);
+        }
+        const double pq = total((double)pc * (double)q, 0);
+        if (!(pq > 0.0)) break;
+        const T alpha = (T)(rz / pq);
+        x = fmadd(alpha, pc, x);
+        r = fmadd(-alpha, q, r);
+        const double rz1 = total((double)r * (double)(r * id), 1);
+        if (rz1 <= stop) break;
+        if (rz1 < best) {
+            best = rz1;
+            since = 0;
+        } else if (++since >= 200) {
+            break;
+        }
+        const T beta = (T)(rz1 / rz);
+        rz = rz1;
+        pc = fmadd(beta, pc, r * id);
+        if (on) p[c] = pc;
+        cl.sync();
+    }
+    if (on) B.phi[c] = x;
+}
+
 // ----------------------------------------------------------- launchers ----
 
 static inline dim3 block2d() { return dim3(kTX, kTY); }
@@ -3703,26 +3805,49 @@ template int cg_bottom_ctas_per_sm<float>();
 
 template <class T>
 cudaError_t launch_cg_bottom(const BoxSet<T> &S, const int *active, T *p, T *q, double *part,
-                             const GridSync &g, int grid, double tol, int maxit, cudaStream_t st)
+                             const GridSync &g, int grid, double tol, int maxit, cudaStream_t st,
+                             bool cluster)
 {
     if (S.nbox == 0 || grid < 1) return cudaSuccess;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = block2d();
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (cluster) {
+        auto *const k = k_cg_bottom_cluster<T>;
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+        cfg.gridDim = dim3(kCgCtas);
+        cfg.blockDim = dim3(kTX, kTY, (S.ntiles[TK_CELL] + kCgCtas - 1) / kCgCtas);
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kCgCtas;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        return counted(cudaLaunchKernelEx(&cfg, k, S, active, p, tol, maxit));
+    }
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = block2d();
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
     return counted(cudaLaunchKernelEx(&cfg, k_cg_bottom<T>, S, active, p, q, part, g, tol, maxit));
 }
 template cudaError_t launch_cg_bottom<double>(const BoxSet<double> &, const int *, double *,
                                               double *, double *, const GridSync &, int, double,
-                                              int, cudaStream_t);
+                                              int, cudaStream_t, bool);
 template cudaError_t launch_cg_bottom<float>(const BoxSet<float> &, const int *, float *, float *,
                                              double *, const GridSync &, int, double, int,
-                                             cudaStream_t);
+                                             cudaStream_t, bool);
+
+// The cluster takes levels of at most kCgCtas x kCgGroups tiles (a thread a
+// cell; see the kernel) where a cluster of that size can be resident.
+template <class T>
+bool cg_cluster_fits(long long tiles)
+{
+    return tiles <= kCgCtas * kCgGroups && tail_clusters<T>(kCgCtas, kTailSmem) > 0;
+}
+template bool cg_cluster_fits<double>(long long);
+template bool cg_cluster_fits<float>(long long);
 
 template <class T>
 cudaError_t launch_guard_fill(const BoxSet<T> &S, T v, cudaStream_t st)

@@ -197,7 +197,12 @@ template <class T>
 int cg_bottom_ctas_per_sm();
 template <class T>
 cudaError_t launch_cg_bottom(const BoxSet<T> &S, const int *active, T *p, T *q, double *part,
-                             const GridSync &g, int grid, double tol, int maxit, cudaStream_t st);
+                             const GridSync &g, int grid, double tol, int maxit, cudaStream_t st,
+                             bool cluster);
+// cluster: by one thread-block cluster instead (the same bits), for levels of
+// few enough cell tiles; q, part and g are then not used.
+template <class T>
+bool cg_cluster_fits(long long tiles);
 
 // ---- moving data between packed user arrays and the level layout --------
 // user[off[b] + (k*ny + j)*nx + i] -> level 0 f (to_f) or phi of box b.

@@ -661,6 +661,9 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
         const auto &db = s->dims[0][s->nlev[0] - 1];
         H.cggrid = std::max(1, std::min({cg_bottom_ctas_per_sm<T>() * s->sms, kCgPartials,
                                          tiles_of(TK_CELL, db[0], db[1], db[2])}));
+        // (a launch whose waits are to give up at once keeps the barrier that can)
+        H.cgcl = s->opts.wait_limit >= 0 && H.cggrid == tiles_of(TK_CELL, db[0], db[1], db[2]) &&
+                 cg_cluster_fits<T>(H.cggrid);
     }
     if (s->opts.persistent) {
         int per_sm = level_ctas_per_sm<T>();
@@ -1783,7 +1786,7 @@ static cudaError_t enqueue_vcycle(Solver *s, const Hier<T> &H, cudaStream_t st,
         e = launch_cg_bottom(H.bottom, s->active, H.cgp, H.cgq, s->cgpart,
                              GridSync{s->gbar, s->derr, sweep_wait_polls(s->opts.wait_limit)},
                              H.cggrid, sizeof(T) == sizeof(double) ? kCgTol64 : kCgTol32,
-                             sizeof(T) == sizeof(double) ? kCgMaxIt64 : kCgMaxIt32, st);
+                             sizeof(T) == sizeof(double) ? kCgMaxIt64 : kCgMaxIt32, st, H.cgcl);
     else
         // (a hierarchy that starts in the kernel starts from the iterate)
         e = launch_coarse_vcycle(H.jobs, H.njobs, H.tail_cl, H.tail_smem, s->active, s->opts.nu1,

@@ -50,6 +50,7 @@ struct Hier {
     int pgrid = 0;                              // resident CTAs of the persistent level kernels
     T *cgp = nullptr, *cgq = nullptr;           // CG coarsest level: p and q (level arrays)
     int cggrid = 0;                             // CG coarsest level: CTAs of its launch
+    bool cgcl = false;                          // CG coarsest level: by one cluster
 };
 
 // A timed stretch of one stage class: events recorded before and after it.

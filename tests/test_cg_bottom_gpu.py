@@ -67,3 +67,23 @@ def test_large_coarsest_level_is_deterministic(cuda_device):
         a, _ = s.solve(f, tol=TOL)
         b, _ = s.solve(f, tol=TOL)
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("shape", [(13, 9, 9), (1, 33, 33), (17, 15, 15), (31, 17, 15), (32, 17, 15),
+                                   (33, 17, 15)])
+def test_cluster_and_grid_launches_match_the_oracle(cuda_device, shape, precision):
+    # 255-cell planes are one tile each: 31 and 32 tiles fill the cluster form's
+    # 16 CTAs of 2 groups but one and fully, 33 take the grid form; 13, 5 and 17
+    # tiles leave CTAs without one or start a second group.  The coarsest level
+    # is the whole box, so the solution is the CG's, held to the bar of the
+    # other shapes.
+    nz, ny, nx = shape
+    d = inputs.stellar((nx, ny, nz), 63)
+    with Solver(shape, d["dx"], precision=precision, device=cuda_device) as s:
+        assert np.prod(s.levels()[-1]) > 1024
+        s.set_beta(_dev(d["beta"], cuda_device))
+        phi, st = s.solve(_dev(d["f"], cuda_device), tol=TOL)
+    assert st["status"] == "ok", st
+    r = O.residual(O.face_beta(d["beta"]), d["dx"], d["f"], phi.cpu().numpy())
+    assert np.linalg.norm(r) <= 1.01 * TOL * np.linalg.norm(d["f"])
