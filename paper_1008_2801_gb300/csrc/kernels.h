@@ -153,6 +153,11 @@ cudaError_t launch_refine_residual(const BoxSet<double> &S64, const BoxSet<float
 cudaError_t launch_judge(int nbox, const double *norm, const double *normf, int *active,
                          const JudgeState &J, cudaGraphConditionalHandle handle, int use_handle,
                          cudaStream_t st);
+// The norm of a set of one box (index 0) from the look-ahead pass's partials,
+// and the decision on it, in one launch (inside the graph of handle).
+cudaError_t launch_norm_judge(const BoxSet<double> &S, const double *partials, double *norm,
+                              const double *normf, int *active, const JudgeState &J,
+                              cudaGraphConditionalHandle handle, cudaStream_t st);
 
 // ---- persistent level sweeps (one launch per level and direction) -------
 // Bounded grid-wide barrier of a persistent launch: `word` (device, zero when

@@ -1845,7 +1845,7 @@ static cudaError_t enqueue_step64(Solver *s, cudaStream_t st)
 
 // Look-ahead head: the finest level's first red pass, out of place, whose
 // partial sums give the residual norm of the iterate it starts from.
-static cudaError_t enqueue_head64(Solver *s, cudaStream_t st)
+static cudaError_t enqueue_look64(Solver *s, cudaStream_t st)
 {
     const BoxSet<double> &S = s->h64.smooth[0];
     int sl = prof_begin(s, MG_PROF_PASS, st);
@@ -1856,7 +1856,16 @@ static cudaError_t enqueue_head64(Solver *s, cudaStream_t st)
     e = launch_rbgs_pass_oop(S, s->active, 0, 0, s->partials, st);
     if (e != cudaSuccess) return e;
     prof_end(s, sl, st);
-    sl = prof_begin(s, MG_PROF_NORM, st);
+    return cudaSuccess;
+}
+
+// The pass and the norm from its sums.
+static cudaError_t enqueue_head64(Solver *s, cudaStream_t st)
+{
+    const BoxSet<double> &S = s->h64.smooth[0];
+    cudaError_t e = enqueue_look64(s, st);
+    if (e != cudaSuccess) return e;
+    const int sl = prof_begin(s, MG_PROF_NORM, st);
     e = launch_norm_finish(S, s->active, s->partials, s->dnorm, nullptr, nullptr, st, nullptr, 2);
     if (e == cudaSuccess) e = combine(s, s->dnorm, st);
     prof_end(s, sl, st);
@@ -2017,7 +2026,14 @@ static cudaError_t enqueue_body64(Solver *s, cudaStream_t st, cudaGraphCondition
 {
     cudaError_t e;
     if (s->lookahead) {
-        if ((e = enqueue_head64(s, st)) != cudaSuccess) return e;
+        const bool one = s->nbox == 1 && !s->coupled;
+        if ((e = (one ? enqueue_look64(s, st) : enqueue_head64(s, st))) != cudaSuccess) return e;
+        if (one) {
+            if ((e = launch_norm_judge(s->h64.smooth[0], s->partials, s->dnorm, s->dnormf,
+                                       s->active, s->J, h, st)) != cudaSuccess)
+                return e;
+            return enqueue_tail64(s, st);
+        }
         if ((e = launch_judge(s->nbox, s->dnorm, s->dnormf, s->active, s->J, h, 1, st)) !=
             cudaSuccess)
             return e;

@@ -11,7 +11,7 @@ import pytest
 import torch
 
 import oracle as O
-from paper_1008_2801_gb300 import LevelSolver, Solver, inputs
+from paper_1008_2801_gb300 import LevelSolver, MGError, Solver, inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -57,3 +57,35 @@ def test_folded_red_pass_on_a_coupled_level(cuda_device):
     s.close()
     ref, _ = O.solve(d["beta"], d["f"], d["dx"], tol=1e-13)
     assert np.linalg.norm(got - ref) <= 1e-9 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("kind", ["nan", "inf", "stall", "zero", "tiny"])
+def test_fused_norm_and_decision_match_the_host_loop(cuda_device, kind):
+    # a single box's device loop forms the norm and decides in one launch; the
+    # host-judged loop in two.  Both add the same partials in the same order, so
+    # every outcome and the history agree bit for bit.
+    shape = (16, 16, 16) if kind == "tiny" else (40, 48, 72)
+    nz, ny, nx = shape
+    d = inputs.stellar((nx, ny, nz), 35)
+    f = np.array(d["f"])
+    if kind in ("nan", "inf"):
+        f[nz // 2, 3, 5] = np.nan if kind == "nan" else np.inf
+    if kind == "zero":
+        f[:] = 0.0
+    out = []
+    for prof in (False, True):
+        with Solver(shape, d["dx"], device=cuda_device) as s:
+            s.profile(prof)
+            s.set_beta(torch.from_numpy(np.array(d["beta"])).to(cuda_device))
+            try:
+                phi, st = s.solve(torch.from_numpy(f).to(cuda_device),
+                                  tol=1e-30 if kind == "stall" else 1e-10)
+            except MGError as e:   # (a non-finite right-hand side is an error)
+                assert kind in ("nan", "inf")
+                out.append((np.zeros(1), dict(status=e.name, cycles=0, hist=[])))
+                continue
+            out.append((phi.cpu().numpy(), st))
+    (a, sa), (b, sb) = out
+    assert np.array_equal(a, b, equal_nan=True)
+    assert sa["status"] == sb["status"] and sa["cycles"] == sb["cycles"]
+    assert np.array_equal(sa["hist"], sb["hist"], equal_nan=True)
