@@ -195,8 +195,8 @@ __device__ __forceinline__ double rcp64(double d)
 // Tile of this CTA in a launch that runs its tiles backwards.  Consecutive
 // kernels of a level alternate direction (red passes, restrictions and the
 // norm pass forwards, black passes and prolongations backwards), so that each
-// starts on what the one before left in L2 (126 MB; a batch of 64 boxes of 64^3
-// takes 29.6 ms against 30.6 with every kernel forwards, a 256^3 solve
+// starts on what the one before left in L2 (126 MB; 64 boxes of 32 to 128 a side
+// take 29.6 ms against 30.6 with every kernel forwards, a 256^3 solve
 // 16.56 against 16.8, 512^3, where L2 holds a twentieth of a pass, 130.0
 // against 130.2).  No kernel reads what another tile of its own launch wrote.
 __device__ __forceinline__ int tile_dir(bool back)

@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
     const int ntile = S.ntiles[TK_SWEEP];
     // t-th tile of this launch in the set's TK_SWEEP index space, taken backwards
     // when the source is phi2 (the sweep before, from phi, ran forwards and ended
-    // with these tiles in L2: a batch of 64 boxes of 64^3 15.67 -> 15.47 ms, 256^3
+    // with these tiles in L2: 64 boxes of 32 to 128 a side 15.67 -> 15.47 ms, 256^3
     // 8.44 -> 8.40, the same at 512^3);
     // the box it belongs to is skipped when it is not active
     struct Tile {
