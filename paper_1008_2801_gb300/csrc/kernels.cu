@@ -1138,6 +1138,8 @@ __global__ void __launch_bounds__(kTailThreads, 1)
     }
     pdl_wait();
     if (active && !active[J.box]) return;  // uniform over the cluster
+    // (the zeros of one thread lie under cells that another copies)
+    if (!zero_start) __syncthreads();
     {   // the first level's f (and phi unless it is 0)
         const Box<T> &B = J.lv[0];
         const TailView<T> V = views[0];

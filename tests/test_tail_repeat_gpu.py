@@ -1,0 +1,77 @@
+"""The coarse V-cycle's cluster kernel where its stages' order hangs on a
+barrier: repeated solves give the same bits (GPU).
+
+A stage that overtakes another changes the iterate, and the number of repeats
+gives it room to; every sum of the solver is taken in a fixed order, so nothing
+else differs between two solves.
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_1008_2801_gb300 import BatchSolver, Solver, inputs
+
+pytestmark = pytest.mark.gpu
+
+REPEATS = 50
+
+
+def _same(solve):
+    first, st0 = solve()
+    first = first.clone()
+    for _ in range(REPEATS - 1):
+        phi, st = solve()
+        assert torch.equal(phi, first) and st == st0
+    return first
+
+
+def _histories(st):
+    return [(x["status"], x["cycles"], x["hist"]) for x in (st if isinstance(st, list) else [st])]
+
+
+# boxes whose finest level runs in the kernel: each cycle there starts from the
+# iterate, which is copied over the zeros that other threads wrote
+@pytest.mark.parametrize("shape,kw", [((8, 8, 8), dict()), ((16, 16, 16), dict(precision="mixed")),
+                                      ((16, 16, 16), dict(coarse_cells=4096)),
+                                      ((8, 8, 8), dict(bc="PPPPDD")),
+                                      ((8, 8, 8), dict(krylov=True))],
+                         ids=["fp64", "mixed", "split", "periodic", "krylov"])
+def test_box_that_starts_in_the_kernel(cuda_device, shape, kw):
+    nz, ny, nx = shape
+    d = inputs.stellar((nx, ny, nz), 41)
+    f = torch.from_numpy(d["f"]).to(cuda_device)
+    with Solver(shape, d["dx"], device=cuda_device, **kw) as s:
+        s.set_beta(torch.from_numpy(d["beta"]).to(cuda_device))
+
+        def solve():
+            phi, st = s.solve(f, tol=1e-10)
+            return phi, _histories(st)
+
+        _same(solve)
+
+
+@pytest.mark.parametrize("precision,small", [("fp64", 8), ("mixed", 16)])
+def test_batch_with_a_box_that_starts_in_the_kernel(cuda_device, precision, small):
+    # one such box among boxes whose coarse levels start from zero; every box is
+    # solved independently, so its bits are those of a batch without the others
+    dims = [(64, 64, 64), (small,) * 3, (32, 64, 48), (64, 64, 64)]
+    data = [inputs.stellar(n, 43 + i) for i, n in enumerate(dims)]
+
+    def batch(which):
+        shapes = [tuple(int(v) for v in dims[i][::-1]) for i in which]
+        s = BatchSolver(shapes, 1 / 64, precision=precision, device=cuda_device,
+                        inner_cycles=2)   # (the adaptive count is one of the whole batch)
+        s.set_beta(s.pack([torch.from_numpy(data[i]["beta"]).to(cuda_device) for i in which]))
+        f = s.pack([torch.from_numpy(data[i]["f"]).to(cuda_device) for i in which])
+
+        def solve():
+            phi, st = s.solve(f, tol=1e-10)
+            return phi, _histories(st)
+
+        phi = _same(solve)
+        out = [a.cpu().numpy() for a in s.unpack(phi)]
+        s.close()
+        return out
+
+    together, small_alone = batch([0, 1, 2, 3]), batch([1, 1, 1, 1])
+    assert np.array_equal(together[1], small_alone[0])
