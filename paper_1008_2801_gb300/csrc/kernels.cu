@@ -1268,6 +1268,9 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         // coarse cell may sit in different CTAs there.
         const Box<T> &B = J.lv[l];
         const bool red = J.tl[l].red != 0, away = l == nd - 1;
+        // (the first CTA may still read the scratch for the level above: with
+        // pre-smoothing, a pass's barrier lies between)
+        if (away && nu1 == 0 && l > 0) cl.sync();
         T *const res = away ? cl.map_shared_rank(sm + J.scratch, 0) : sm + J.scratch;
         const int kb = away ? V.z0 : 0, nr = red ? V.nx >> 1 : V.nx;
         const T *const gd = B.D;
