@@ -552,7 +552,12 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
     std::vector<CoarseJob<T>> jobs;
     const long long lim = coarse_limit<T>(s->opts);
     H.lc.assign(s->nbox, 0);
-    H.tail_cl = lim > 0 && !s->cg_bottom && !s->coupled ? tail_cluster<T>(s->nbox) : 1;
+    H.tail_cl = 1;
+    if (!s->cg_bottom && !s->coupled) {
+        if (lim > 0) H.tail_cl = tail_cluster<T>(s->nbox);
+        else tail_clusters<T>(1, kTailSmem);   // (the coarsest level alone: a thin one of 1024
+                                               // cells takes 82 KB of shared memory)
+    }
     H.tail_smem = 0;
     for (int b = 0; b < s->nbox; ++b) {
         fine.push_back(make_box(s, H, b, 0));
