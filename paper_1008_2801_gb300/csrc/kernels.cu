@@ -1137,7 +1137,10 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         for (int q = tid; q < n * n; q += kTailThreads) tail_async<1>(sm + J.ainv + q, B.ainv + q);
     }
     pdl_wait();
-    if (active && !active[J.box]) return;  // uniform over the cluster
+    if (active && !active[J.box]) {        // uniform over the cluster
+        tail_async_wait();                 // (no copy may land after the CTA has gone)
+        return;
+    }
     // (the zeros of one thread lie under cells that another copies)
     if (!zero_start) __syncthreads();
     {   // the first level's f (and phi unless it is 0)

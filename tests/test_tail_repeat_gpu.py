@@ -101,3 +101,33 @@ def test_no_pre_smoothing_over_two_split_levels(cuda_device, shape, kw):
             return phi, _histories(st)
 
         assert torch.equal(_same(solve), ref)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_boxes_that_stop_at_different_cycles(cuda_device, precision):
+    # a box that is done leaves the kernel with its weights' copies in flight
+    # while the others run; each box's bits are those of its own solve
+    d = inputs.batched(24, 53, sizes=(16, 24, 32, 48), dx=1 / 48)
+    shapes = [tuple(int(v) for v in n[::-1]) for n in d["dims"]]
+
+    def batch(which):
+        s = BatchSolver([shapes[i] for i in which], d["dx"], precision=precision,
+                        device=cuda_device, inner_cycles=2)
+        s.set_beta(s.pack([torch.from_numpy(d["beta"][i]).to(cuda_device) for i in which]))
+        f = s.pack([torch.from_numpy(d["f"][i]).to(cuda_device) for i in which])
+
+        def solve():
+            phi, st = s.solve(f, tol=1e-10)
+            return phi, _histories(st)
+
+        phi, cycles = _same(solve), [c for _, c, _ in solve()[1]]
+        out = [a.clone() for a in s.unpack(phi)]
+        s.close()
+        return out, cycles
+
+    together, cycles = batch(range(24))
+    if precision == "fp64":
+        assert len(set(cycles)) > 1
+    for i in range(0, 24, 5):
+        alone, _ = batch([i])
+        assert torch.equal(together[i], alone[0])
