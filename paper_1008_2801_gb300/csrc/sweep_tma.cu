@@ -34,7 +34,10 @@
 // Waits are bounded: a wait that gives up sets the error word and the
 // threads go on (no consumer may leave the loop while the others meet at
 // the named barrier); the producer stops issuing, and before it exits it
-// waits, with the default bound, for every copy it issued.
+// waits, with the default bound, for every copy it issued.  A consumer that
+// gave up says so in shared memory before it releases another stage: the plane
+// there may still be landing, and a copy into it would open the next phase of
+// its barrier over the one in flight.
 //
 // TMA rules kept: every copy starts at x = x0 - 4 (x0 a multiple of 32), a
 // multiple of 4 floats = 16 bytes; rows are P floats with P a multiple of 8;
@@ -231,6 +234,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
     float *const sm = reinterpret_cast<float *>(smem);
     float *const red = sm + NS * STG;
     __shared__ __align__(8) unsigned long long full[NS], empty[NS];
+    __shared__ volatile int gave_up;
 
     const int *ts = S.tstart[TK_SWEEP];
     const int ntile = S.ntiles[TK_SWEEP];
@@ -260,6 +264,7 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
     };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
+        gave_up = 0;
         for (int s = 0; s < NS; ++s) {
             mbar_init(smem_addr(&full[s]), 1);
             mbar_init(smem_addr(&empty[s]), kConsumers);
@@ -304,7 +309,8 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
                         if (tn < ntile && N.b != T.b) acquire(N.b);
                     }
                     if (i >= NS &&
-                        !mbar_wait(smem_addr(&empty[s]), (unsigned)(((i / NS) - 1) & 1), polls)) {
+                        (!mbar_wait(smem_addr(&empty[s]), (unsigned)(((i / NS) - 1) & 1), polls) ||
+                         gave_up)) {
                         atomicExch(err, 1);
                         ok = false;
                         break;
@@ -341,7 +347,8 @@ __global__ void __launch_bounds__(kTmaThreads, MINB)
     auto take = [&]() {   // the next plane's stage, once the plane has landed in it
         const int st = rg.s;
         if (!mbar_wait(smem_addr(&full[st]), rg.par, left)) {
-            if (lane == 0) atomicExch(err, 1);
+            atomicExch(err, 1);
+            gave_up = 1;
             left = 0;     // (a wait that gave up is not repeated)
         }
         rg.next();

@@ -1,0 +1,33 @@
+"""Short limits on device waits: a solve ends in its result or in a timeout, and
+the device stays usable (GPU)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1008_2801_gb300 import MGError, Solver, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [(128, 64, 64), (96, 48, 80)])   # 64- and 32-wide tiles
+@pytest.mark.parametrize("limit", [1, 2, 3, 50, 2000])
+def test_tile_copy_waits(cuda_device, n, limit):
+    # after a consumer gave up the producer issues no further copy: no solve may
+    # end in other bits than the default bound's
+    d = inputs.stellar(n, 57)
+    beta, f = (torch.from_numpy(d[k]).to(cuda_device) for k in ("beta", "f"))
+    kw = dict(precision="mixed", smoother="fused", tma=True, device=cuda_device)
+    with Solver(f.shape, d["dx"], **kw) as s:
+        s.set_beta(beta)
+        ref, _ = s.solve(f, tol=1e-10)
+        with Solver(f.shape, d["dx"], wait_limit=limit, **kw) as q:
+            q.set_beta(beta)
+            for _ in range(20):
+                try:
+                    phi, _ = q.solve(f, tol=1e-10)
+                except MGError as e:
+                    assert e.name == "timeout"
+                else:
+                    assert torch.equal(phi, ref)
+        again, _ = s.solve(f, tol=1e-10)
+    assert torch.equal(again, ref)
