@@ -159,9 +159,13 @@ typedef struct {
     int max_norm;     /* 1: also report rel_resid_max in mg_stats (one more
                          pass over the level after the solve); 0 (default) */
     int wait_limit;   /* bounded device waits (the TMA sweep's tile-copy
-                         waits): polls of the barrier before a wait gives
+                         waits, the grid barriers of persistent launches and
+                         of the CG solve of a large coarsest level): polls of
+                         the barrier before a wait gives
                          up, sets the context's error word and the solve
-                         returns MG_ERR_TIMEOUT.  0 (default): 2^22 polls;
+                         returns MG_ERR_TIMEOUT.  0 (default): 2^22 polls,
+                         and CG solves of few tiles run in one thread-block
+                         cluster, whose hardware barriers poll nothing;
                          n > 0: n polls; -1: give up at the first wait
                          (exercises the timeout path; the CTA still drains
                          the copies it issued before it exits) */

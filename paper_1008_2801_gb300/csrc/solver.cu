@@ -666,8 +666,8 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
         const auto &db = s->dims[0][s->nlev[0] - 1];
         H.cggrid = std::max(1, std::min({cg_bottom_ctas_per_sm<T>() * s->sms, kCgPartials,
                                          tiles_of(TK_CELL, db[0], db[1], db[2])}));
-        // (a launch whose waits are to give up at once keeps the barrier that can)
-        H.cgcl = s->opts.wait_limit >= 0 && H.cggrid == tiles_of(TK_CELL, db[0], db[1], db[2]) &&
+        // (a caller who limits the waits gets the barrier that can give up)
+        H.cgcl = s->opts.wait_limit == 0 && H.cggrid == tiles_of(TK_CELL, db[0], db[1], db[2]) &&
                  cg_cluster_fits<T>(H.cggrid);
     }
     if (s->opts.persistent) {

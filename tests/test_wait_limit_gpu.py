@@ -1,6 +1,5 @@
 """Short limits on device waits: a solve ends in its result or in a timeout, and
 the device stays usable (GPU)."""
-import numpy as np
 import pytest
 import torch
 
@@ -31,3 +30,26 @@ def test_tile_copy_waits(cuda_device, n, limit):
                     assert torch.equal(phi, ref)
         again, _ = s.solve(f, tol=1e-10)
     assert torch.equal(again, ref)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_limit_on_the_cg_coarsest_solve(cuda_device, precision):
+    # 13 tiles of 9 x 9 cells: one cluster by default, a limit takes the grid
+    # barrier.  One poll does not see thirteen CTAs through some hundred barriers;
+    # a large number does, with the default form's bits.
+    d = inputs.stellar((9, 9, 13), 59)
+    beta, f = (torch.from_numpy(d[k]).to(cuda_device) for k in ("beta", "f"))
+    kw = dict(precision=precision, device=cuda_device)
+    out = []
+    for limit in (0, 1 << 20):
+        with Solver(f.shape, d["dx"], wait_limit=limit, **kw) as s:
+            s.set_beta(beta)
+            phi, st = s.solve(f, tol=1e-10)
+            assert st["status"] == "ok"
+            out.append(phi)
+    assert torch.equal(*out)
+    with Solver(f.shape, d["dx"], wait_limit=1, **kw) as s:
+        s.set_beta(beta)
+        with pytest.raises(MGError) as ei:
+            s.solve(f, tol=1e-10)
+        assert ei.value.name == "timeout"
