@@ -12,6 +12,8 @@
 // guarded level layout described in common.cuh.
 #include "kernels.h"
 
+#include "cluster.h"
+
 #include <algorithm>
 #include <cooperative_groups.h>
 #include <type_traits>
@@ -3482,19 +3484,20 @@ cudaError_t launch_bottom(const BoxSet<T> &S, const int *active, int max_cells, 
     return counted(cudaGetLastError());
 }
 
-template <class T>
-int tail_clusters(int cl, size_t smem)
+// Clusters of cl CTAs of a kernel that can be resident at once (0: none); also
+// allows the kernel such clusters and smem bytes of dynamic shared memory.
+template <class K>
+static int resident_clusters(K *k, int cl, dim3 block, size_t smem)
 {
-    void (*const k)(const CoarseJob<T> *, const int *, int, int, int, int) = k_coarse_vcycle<T>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmem) !=
-            cudaSuccess) {
+        (smem > 0 && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)smem) != cudaSuccess)) {
         cudaGetLastError();
         return 0;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cl);
-    cfg.blockDim = dim3(kTailThreads);
+    cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -3509,6 +3512,12 @@ int tail_clusters(int cl, size_t smem)
         return 0;
     }
     return n;
+}
+
+template <class T>
+int tail_clusters(int cl, size_t smem)
+{
+    return resident_clusters(k_coarse_vcycle<T>, cl, dim3(kTailThreads), smem);
 }
 template int tail_clusters<double>(int, size_t);
 template int tail_clusters<float>(int, size_t);
@@ -3648,10 +3657,30 @@ cudaError_t launch_round_f32(int nx, int ny, int nz, const double *wx, const dou
 // CTAs of the cluster that inverts an n x n matrix (nbox of them at once), and
 // the shared memory of each: short matrices are a chain of barriers, which one
 // CTA passes fastest.
-static int inv_ctas(int n, int nbox)
+static int inv_ctas(int n, int nbox, int limit)
 {
-    int c = n >= 128 ? 16 : n >= 48 ? 8 : 1;
-    while (c > 1 && (long long)c * nbox > 304) c /= 2;   // (two waves of CTAs)
+    const int c = std::min(n >= 128 ? 16 : n >= 48 ? 8 : 1, limit);
+    return cluster_step_down(c, [&](int k) { return (long long)k * nbox <= 304; });   // (two waves)
+}
+// The largest cluster of an inverse kernel that the current device can hold
+// with the most shared memory it takes; asked once a device.
+template <class K>
+static int inv_limit(K *kernel, int which)
+{
+    constexpr int kMaxDevices = 64;
+    static std::mutex mu;
+    static int known[3][kMaxDevices] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+        cudaGetLastError();
+        dev = -1;
+    }
+    std::lock_guard<std::mutex> lk(mu);
+    if (dev >= 0 && known[which][dev]) return known[which][dev];
+    const int c = cluster_step_down(16, [&](int k) {
+        return resident_clusters(kernel, k, dim3(kInvThreads), kTailSmem) > 0;
+    });
+    if (dev >= 0) known[which][dev] = c;
     return c;
 }
 static int inv_bytes(int n, int ctas, bool fp64)
@@ -3686,7 +3715,8 @@ cudaError_t launch_bottom_inverse(int nx, int ny, int nz, const double *wx, cons
                                   const double *wz, int singular, double *work, double *inv64,
                                   float *inv32, cudaStream_t st)
 {
-    const int n = nx * ny * nz, c = inv_ctas(n, 1), smem = inv_bytes(n, c, true);
+    const int n = nx * ny * nz, c = inv_ctas(n, 1, inv_limit(k_bottom_inverse, 0)),
+              smem = inv_bytes(n, c, true);
     return inv_launch(k_bottom_inverse, 1, c, smem, st, nx, ny, nz, (int)pitch_row(nx),
                       (long long)pitch_plane(nx, ny), wx, wy, wz, singular, work, inv64, inv32, smem);
 }
@@ -3719,7 +3749,8 @@ cudaError_t launch_setup(const SetupSet &S, int step, cudaStream_t st)
 cudaError_t launch_setup_bottom(const SetupSet &S, int max_cells, bool fp64, cudaStream_t st)
 {
     if (S.nbox == 0) return cudaSuccess;
-    const int c = inv_ctas(max_cells, S.nbox), smem = inv_bytes(max_cells, c, fp64);
+    const int c = inv_ctas(max_cells, S.nbox, inv_limit(k_setup_bottom, 1)),
+              smem = inv_bytes(max_cells, c, fp64);
     return inv_launch(k_setup_bottom, S.nbox, c, smem, st, S, smem);
 }
 
@@ -3911,7 +3942,8 @@ cudaError_t launch_guard_fill(const BoxSet<T> &S, T v, cudaStream_t st)
 cudaError_t launch_union_inverse(const SetupSet &S, const UnionBottom &U, double *work,
                                  double *inv64, float *inv32, cudaStream_t st)
 {
-    const int c = inv_ctas(U.n, 1), smem = inv_bytes(U.n, c, true);
+    const int c = inv_ctas(U.n, 1, inv_limit(k_union_inverse, 2)),
+              smem = inv_bytes(U.n, c, true);
     return inv_launch(k_union_inverse, 1, c, smem, st, S, U, work, inv64, inv32, smem);
 }
 

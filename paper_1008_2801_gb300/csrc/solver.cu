@@ -8,6 +8,8 @@
 // fine-level residual norm) is captured once as a CUDA graph and replayed.
 #include "solver.h"
 
+#include "cluster.h"
+
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -497,10 +499,10 @@ static size_t plan_tail(const Solver *s, int b, int lc, int cl, CoarseJob<T> *J)
 template <class T>
 static int tail_cluster(int nbox)
 {
-    for (int cl = 16; cl > 1; cl /= 2)
-        if (tail_clusters<T>(cl, kTailSmem) >= nbox) return cl;
-    tail_clusters<T>(1, kTailSmem);
-    return 1;
+    const int cl = cluster_step_down(
+        16, [&](int c) { return tail_clusters<T>(c, kTailSmem) >= nbox; });
+    if (cl == 1) tail_clusters<T>(1, kTailSmem);
+    return cl;
 }
 
 // A level joins the cluster's part while a pass over it costs less there than
