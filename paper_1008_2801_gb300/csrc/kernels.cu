@@ -3926,7 +3926,8 @@ template cudaError_t launch_cg_bottom<float>(const BoxSet<float> &, const int *,
 template <class T>
 bool cg_cluster_fits(long long tiles)
 {
-    return tiles <= kCgCtas * kCgGroups && tail_clusters<T>(kCgCtas, kTailSmem) > 0;
+    return tiles <= kCgCtas * kCgGroups &&
+           resident_clusters(k_cg_bottom_cluster<T>, kCgCtas, dim3(kTX, kTY, kCgGroups), 0) > 0;
 }
 template bool cg_cluster_fits<double>(long long);
 template bool cg_cluster_fits<float>(long long);
