@@ -284,6 +284,7 @@ struct CoarseJob {
     int ndist;
     int nzc;        // planes of level ndist - 1 (the coarsest split level)
     int per;        // bits 0-2: x, y, z axis periodic
+    int zero;       // phi of lv[0] is 0 on entry (it is not read)
     int scratch;    // offset: residuals of the coarsest split level (first CTA)
     int ainv;       // offset: dense coarsest inverse (first CTA), -1: in global memory
     TailLevel tl[kMaxCoarse];

@@ -1037,7 +1037,7 @@ __device__ __forceinline__ void tail_push(const cg::cluster_group &cl, const Tai
 template <class T>
 __global__ void __launch_bounds__(kTailThreads, 1)
     k_coarse_vcycle(const CoarseJob<T> *__restrict__ jobs, const int *__restrict__ active, int nu1,
-                    int nu2, int post_first, int zero_start)
+                    int nu2, int post_first)
 {
     extern __shared__ __align__(16) char tail_smem[];
     __shared__ CoarseJob<T> J;
@@ -1054,6 +1054,7 @@ __global__ void __launch_bounds__(kTailThreads, 1)
     }
     __syncthreads();
     const int nl = J.nlev, nd = J.ndist, per = J.per;
+    const bool zero_start = J.zero != 0;
     if (tid < nl) {   // a thread per level
         const int l = tid;
         const Box<T> &B = J.lv[l];
@@ -3525,7 +3526,7 @@ template int tail_clusters<float>(int, size_t);
 template <class T>
 cudaError_t launch_coarse_vcycle(const CoarseJob<T> *jobs, int njobs, int cl, size_t smem,
                                  const int *active, int nu1, int nu2, cudaStream_t st,
-                                 int post_first, bool zero_start)
+                                 int post_first)
 {
     if (njobs == 0) return cudaSuccess;
     cudaLaunchConfig_t cfg = {};
@@ -3542,8 +3543,7 @@ cudaError_t launch_coarse_vcycle(const CoarseJob<T> *jobs, int njobs, int cl, si
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = pdl_enabled() ? 2 : 1;
-    return counted(cudaLaunchKernelEx(&cfg, k_coarse_vcycle<T>, jobs, active, nu1, nu2, post_first,
-                                      zero_start ? 1 : 0));
+    return counted(cudaLaunchKernelEx(&cfg, k_coarse_vcycle<T>, jobs, active, nu1, nu2, post_first));
 }
 
 cudaError_t launch_refine_update(const BoxSet<double> &S64, const BoxSet<float> &S32,
@@ -4023,7 +4023,7 @@ cudaError_t launch_pcg_mixed(const BoxSet<double> &S64, const BoxSet<float> &S32
     template cudaError_t launch_bottom<T>(const BoxSet<T> &, const int *, int, cudaStream_t);   \
     template cudaError_t launch_zero<T>(const BoxSet<T> &, const int *, cudaStream_t);          \
     template cudaError_t launch_coarse_vcycle<T>(const CoarseJob<T> *, int, int, size_t,            \
-                                                 const int *, int, int, cudaStream_t, int, bool);   \
+                                                 const int *, int, int, cudaStream_t, int);         \
     template cudaError_t launch_exchange<T>(const BoxSet<T> &, const int *, const ExchRec *, int,  \
                                             int, cudaStream_t, int);                                         \
     template cudaError_t launch_guard_fill<T>(const BoxSet<T> &, T, cudaStream_t);                 \

@@ -127,11 +127,10 @@ cudaError_t launch_bottom(const BoxSet<T> &S, const int *active, int max_cells, 
 // per job, its levels in smem bytes of shared memory a CTA.
 // post_first: colour of the first pass of each post-smoothing sweep (0 red,
 // the default; 1 black: the post-smoother is the pre-smoother's adjoint).
-// zero_start: the first level's phi is 0 on entry (it is not read).
 template <class T>
 cudaError_t launch_coarse_vcycle(const CoarseJob<T> *jobs, int njobs, int cl, size_t smem,
                                  const int *active, int nu1, int nu2, cudaStream_t st,
-                                 int post_first, bool zero_start);
+                                 int post_first);
 // Clusters of cl CTAs with smem bytes each that can be resident at once (0:
 // none); also allows the kernel its cluster size and shared memory.
 template <class T>

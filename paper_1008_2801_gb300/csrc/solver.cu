@@ -585,6 +585,7 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
         }
         H.lc[b] = lc;
         H.tail_smem = std::max(H.tail_smem, plan_tail(s, b, lc, H.tail_cl, &J));
+        J.zero = lc > 0;   // (a box whose finest level it is starts from the iterate)
         for (int l = lc; l < s->nlev[b]; ++l) J.lv[l - lc] = make_box(s, H, b, l);
         jobs.push_back(J);
     }
@@ -663,7 +664,6 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
         H.smooth[l].fold = l + 1 < (int)H.smooth.size() && H.red_done[l + 1];
     }
     H.njobs = (int)jobs.size();
-    H.tail_zero = *std::min_element(H.lc.begin(), H.lc.end()) > 0;
     *jobs_off = blob.put(jobs.data(), jobs.size() * sizeof(CoarseJob<T>));
     if (s->cg_bottom) {
         const auto &db = s->dims[0][s->nlev[0] - 1];
@@ -1796,9 +1796,8 @@ static cudaError_t enqueue_vcycle(Solver *s, const Hier<T> &H, cudaStream_t st,
                              H.cggrid, sizeof(T) == sizeof(double) ? kCgTol64 : kCgTol32,
                              sizeof(T) == sizeof(double) ? kCgMaxIt64 : kCgMaxIt32, st, H.cgcl);
     else
-        // (a hierarchy that starts in the kernel starts from the iterate)
         e = launch_coarse_vcycle(H.jobs, H.njobs, H.tail_cl, H.tail_smem, s->active, s->opts.nu1,
-                                 s->opts.nu2, st, sym ? 1 : 0, H.tail_zero);
+                                 s->opts.nu2, st, sym ? 1 : 0);
     if (e != cudaSuccess) return e;
     for (int l = nl - 1; l >= 0; --l) {
         const BoxSet<T> &S = H.smooth[l];

@@ -41,7 +41,6 @@ struct Hier {
     int njobs = 0;
     int tail_cl = 1;                            // CTAs of a job's cluster
     size_t tail_smem = 0;                       // shared memory of such a CTA
-    bool tail_zero = false;                     // every job's first level starts from phi = 0
     cudaGraphExec_t graph = nullptr;            // captured V-cycle (+ fine norm for FP64)
     cudaGraphExec_t head = nullptr;             // look-ahead: first red pass + norm
     cudaGraphExec_t down0 = nullptr;            // host-judged inner cycles: finest level's down leg

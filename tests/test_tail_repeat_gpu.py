@@ -73,8 +73,10 @@ def test_batch_with_a_box_that_starts_in_the_kernel(cuda_device, precision, smal
         s.close()
         return out
 
-    together, small_alone = batch([0, 1, 2, 3]), batch([1, 1, 1, 1])
+    together, small_alone, large = batch([0, 1, 2, 3]), batch([1, 1, 1, 1]), batch([0, 2, 3])
     assert np.array_equal(together[1], small_alone[0])
+    for i, a in zip((0, 2, 3), large):
+        assert np.array_equal(together[i], a)
 
 
 @pytest.mark.parametrize("shape", [(64, 64, 64), (64, 48, 80)])
