@@ -335,7 +335,7 @@ static SetPlan<D> plan_set(DescBlob &blob, DescSet<D> *target, const std::vector
     p.target = target;
     *target = DescSet<D>{};
     target->nbox = (int)boxes.size();
-    p.boxes_off = blob.put(boxes.data(), boxes.size() * sizeof(D));
+    p.boxes_off = blob.put(boxes.data(), boxes.size() * sizeof(D), 128);   // (see Box)
     for (int k = 0; k < TK_NKIND; ++k) {
         std::vector<int> ts(boxes.size() + 1, 0);
         for (size_t i = 0; i < boxes.size(); ++i) {
