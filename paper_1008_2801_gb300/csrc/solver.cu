@@ -183,6 +183,12 @@ static void carve(Solver *s, Hier<T> &H, Bump &bump, bool full)
             T *pp = bump.take<T>((size_t)E), *qq = bump.take<T>((size_t)E);
             H.cgp = pp ? pp + Q : nullptr;
             H.cgq = qq ? qq + Q : nullptr;
+            // its residual lies in phi2, where outer CG keeps the solution of a
+            // box that is its own coarsest level: that one gets an array
+            if (s->pcg && !s->has32 && s->nlev[b] == 1) {
+                T *rr = bump.take<T>((size_t)E);
+                H.cgr = rr ? rr + Q : nullptr;
+            }
         } else if (!s->xmode) {
             H.ainv[b] = (s->shared && b > 0) ? H.ainv[0] : bump.take<T>(nb * nb);
         }
@@ -564,6 +570,7 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
     for (int b = 0; b < s->nbox; ++b) {
         fine.push_back(make_box(s, H, b, 0));
         bottom.push_back(make_box(s, H, b, s->nlev[b] - 1));
+        if (H.cgr) bottom.back().phi2 = H.cgr;
         // first level of the coarse kernel (the coarsest level always is one:
         // it is solved there when the kernel is off): every level within the
         // limit, then finer ones (never the finest, whose cycle also judges

@@ -48,6 +48,7 @@ struct Hier {
     T *uinv = nullptr;                          // coupled level: dense inverse of the union bottom
     int pgrid = 0;                              // resident CTAs of the persistent level kernels
     T *cgp = nullptr, *cgq = nullptr;           // CG coarsest level: p and q (level arrays)
+    T *cgr = nullptr;                           // ... its residual, unless that may lie in phi2
     int cggrid = 0;                             // CG coarsest level: CTAs of its launch
     bool cgcl = false;                          // CG coarsest level: by one cluster
 };

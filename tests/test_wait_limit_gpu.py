@@ -1,8 +1,10 @@
 """Short limits on device waits: a solve ends in its result or in a timeout, and
 the device stays usable (GPU)."""
+import numpy as np
 import pytest
 import torch
 
+import oracle as O
 from paper_1008_2801_gb300 import MGError, Solver, inputs
 
 pytestmark = pytest.mark.gpu
@@ -53,3 +55,19 @@ def test_limit_on_the_cg_coarsest_solve(cuda_device, precision):
         with pytest.raises(MGError) as ei:
             s.solve(f, tol=1e-10)
         assert ei.value.name == "timeout"
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("shape,limit", [((13, 9, 9), 0), ((13, 9, 9), 1 << 20), ((33, 33, 33), 0)])
+def test_cg_around_a_cg_coarsest_solve(cuda_device, shape, limit, precision):
+    # a box that is its own coarsest level: the outer iteration's solution must
+    # not share an array with the inner one's residual, in either form
+    nz, ny, nx = shape
+    d = inputs.stellar((nx, ny, nz), 59)
+    with Solver(shape, d["dx"], precision=precision, krylov=True, wait_limit=limit,
+                device=cuda_device) as s:
+        s.set_beta(torch.from_numpy(d["beta"]).to(cuda_device))
+        phi, st = s.solve(torch.from_numpy(d["f"]).to(cuda_device), tol=1e-10)
+    assert st["status"] == "ok", st
+    r = O.residual(O.face_beta(d["beta"]), d["dx"], d["f"], phi.cpu().numpy())
+    assert np.linalg.norm(r) <= 1.01e-10 * np.linalg.norm(d["f"])
