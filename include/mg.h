@@ -322,7 +322,7 @@ int mg_levels(const mg_ctx *ctx, int *nlev, int *dims);
 
 /* How the context smooths level `level` of its V-cycles (FP32 levels in
  * mixed precision, else FP64): *kind = 0 single-colour passes (or the
- * level is in the one-CTA coarse kernel, or is the coarsest), 1 fused
+ * level is in the cluster coarse kernel, or is the coarsest), 1 fused
  * sweeps with plain loads, 2 fused sweeps fed by the Tensor Memory
  * Accelerator.  Host only.  INVALID_ARG for a level outside the list. */
 int mg_smoother_kind(const mg_ctx *ctx, int level, int *kind);

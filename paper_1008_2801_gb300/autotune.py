@@ -2,18 +2,18 @@
 and precision.
 
 The library picks its launch shapes from models (the fused sweep's z-chunk
-fills whole waves of resident CTAs; small levels go to the one-CTA coarse
+fills whole waves of resident CTAs; small levels go to the cluster coarse
 kernel; a persistent launch takes as many CTAs as can be resident).  What a
 model cannot know well is where the cross-overs sit on a given GPU for a
 given shape.  ``tune`` searches in two stages on a synthetic stellar-profile
 problem of the requested shape(s):
 
-1. options: fused sweeps or single-colour passes, how many cells the one-CTA
+1. options: fused sweeps or single-colour passes, how many cells the cluster
    coarse kernel takes, (mixed precision) FP32 V-cycles per FP64 refinement
    step, and per-stage launches or one persistent launch per level and
    direction;
 2. tile shapes for the best options: the fused FP32 sweep's tile depth
-   (planes of z per CTA, ``sweep_zc``; its tile is 64 x 8 cells in x, y) and
+   (planes of z per CTA, ``sweep_zc``; its tile is 64 x 8 or 32 x 16 cells in x, y) and
    the persistent launches' CTAs per SM (``level_ctas``).
 
 It keeps the fastest and caches it in a JSON file keyed by GPU name, shape

@@ -198,9 +198,10 @@ __device__ __forceinline__ double rcp64(double d)
 // kernels of a level alternate direction (red passes, restrictions and the
 // norm pass forwards, black passes and prolongations backwards), so that each
 // starts on what the one before left in L2 (126 MB; 64 boxes of 32 to 128 a side
-// take 29.6 ms against 30.6 with every kernel forwards, a 256^3 solve
-// 16.56 against 16.8, 512^3, where L2 holds a twentieth of a pass, 130.0
-// against 130.2).  No kernel reads what another tile of its own launch wrote.
+// take 29.6 ms against 30.6 with every kernel forwards, a 256^3 solve 16.56
+// against 16.8, 128^3 3.05 against 3.07; the same at 512^3, where L2 holds a
+// twentieth of a pass).  Levels that L2 holds whole gain nothing and lose up to
+// 0.05 us a launch (96^3 by launches 2.30 ms against 2.24).  No kernel reads what another tile of its own launch wrote.
 __device__ __forceinline__ int tile_dir(bool back)
 {
     return back ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
@@ -930,7 +931,7 @@ __global__ void __launch_bounds__(kThreads) k_bottom(BoxSet<T> S, const int *__r
 // one cluster barrier ends each pass.  The levels below (at most kTailSolo
 // cells) run in the cluster's first CTA alone, where a block barrier does.
 // What bounds it: the dependent chain of about 20 stages per two levels, each
-// a barrier (~0.3 us), the shared-memory latency and, in FP64, the narrow pipe
+// a barrier (~0.4 us), the shared-memory latency and, in FP64, the narrow pipe
 // (16 cycles an SM per warp instruction: 1.7 us for a pass over 32^3 on 16
 // SMs; a chain of 7 dependent FP64 operations alone is 0.4 us).  Weights are
 // loaded before the wait on the preceding kernel.  FP64, 32^3 and below: 60 us

@@ -652,10 +652,13 @@ static void plan_hier(Solver *s, Hier<T> &H, DescBlob &blob,
             }
         }
         // the level below, where it smooths with passes, takes its first red
-        // pass from this level's restriction (sets of up to 32^3 cells keep a
-        // launch per stage: they are launched only where the cluster kernel is
-        // off or has no place, and the launch counts are read there; slabs run
-        // every pass themselves, 384^3 in two 65.05 ms against 65.32 with the fold)
+        // pass from this level's restriction.  Sets of up to 32^3 cells keep a
+        // launch a stage for the sake of mg_profile.kernels, which is read as ten
+        // launches a small level and cycle, not of time: the fold gains there too
+        // (launched where the cluster kernel is off or has no place: 64^3 FP64 with
+        // coarse_cells = -1 1.75 -> 1.66 ms, 32 coupled boxes of 64^3 14.50 ->
+        // 14.35).  Slabs run every pass themselves (384^3 in two 65.05 ms against
+        // 65.32 with the fold).
         long long below = 0;
         for (const auto &B : set)
             if (l + 1 < H.lc[B.box]) below += (long long)(B.nx / 2) * (B.ny / 2) * (B.nz / 2);
@@ -802,8 +805,8 @@ int solver_create(Solver **out, int nbox, const int (*n)[3], const double *dx, i
         // ghost exchanges between boxes (or across periodic faces) before
         // every stencil: single-colour passes; a coupled level launches
         // every level down to the dense bottom solve of the union (a
-        // periodic box runs its coarse levels in the one-CTA kernel, which
-        // does its own exchanges)
+        // periodic box runs its coarse levels in the cluster kernel, whose
+        // passes store boundary cells into the guard cells that copy them)
         o.smoother = 1;
         if (coupled) o.coarse_cells = -1;
         o.tma = -1;
