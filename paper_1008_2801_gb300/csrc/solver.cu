@@ -2141,6 +2141,7 @@ static int run_loop(Solver *s, cudaGraphExec_t *exec, long long *per_iter, F bod
         np.conditional.type = cudaGraphCondTypeWhile;
         np.conditional.size = 1;
         cudaGraphNode_t node;
+        bool body_lost = false;
         if (e == cudaSuccess) e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &np);
         if (e == cudaSuccess) {
             cudaGraph_t bodyg = np.conditional.phGraph_out[0];
@@ -2153,10 +2154,13 @@ static int run_loop(Solver *s, cudaGraphExec_t *exec, long long *per_iter, F bod
                 s->cap_kernels += *per_iter;
                 cudaError_t ee = cudaStreamEndCapture(s->cap, &bodyg);
                 e = eb != cudaSuccess ? eb : ee;
+                // the driver frees the body of a capture that fails, and
+                // destroying its parent then frees it again and crashes
+                body_lost = e != cudaSuccess;
             }
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(exec, g, 0);
-        cudaGraphDestroy(g);
+        if (!body_lost) cudaGraphDestroy(g);
         if (e != cudaSuccess) {
             *exec = nullptr;
             return set_error(MG_ERR_CUDA, "convergence-loop graph: %s", cudaGetErrorString(e));
